@@ -76,21 +76,6 @@ __device__ __forceinline__ void for_p2(int t, F&& f) {
 
 __device__ __forceinline__ float2 ldg2(const float2* p) { return __ldg(p); }
 
-// The forward model's propagations multiply by the full propagator table
-// (one rounding per element fewer; the residual amplifies the forward
-// model's rounding), the adjoint's by the separable factors in shared memory.
-#ifndef PTYCHO_PROP_TABLE
-#define PTYCHO_PROP_TABLE 1
-#endif
-template <class C>
-__device__ __forceinline__ void mul_prop_fwd(float2 (&v)[C::V], const float2* hs, const float2* h2, int t) {
-#if PTYCHO_PROP_TABLE
-  mul_table<C, false>(v, h2, t);
-#else
-  mul_separable<C, false>(v, hs, t);
-#endif
-}
-
 // Recompute mode's finished patches are read once by the accumulation that
 // follows each launch: streaming stores by default; plain stores (to keep a
 // chunk's patches in L2 when the chunk is small enough) with
@@ -135,8 +120,11 @@ __global__ void __launch_bounds__(Cfg<M>::T, Cfg<M>::MIN_BLOCKS)
 int chain_threads(int M) { return M == 128 ? Cfg<128>::T : Cfg<64>::T; }
 
 size_t chain_smem_bytes(int M) {
-  return (size_t)M * M * sizeof(float2) + 2 * (size_t)M * sizeof(float2) +
-         (size_t)(chain_threads(M) / 32) * sizeof(double);
+  // the exchange buffer, the pass-1 twiddle table, the loss partials of the
+  // warps and the tensor-memory address
+  const size_t tw1 = 16 * (size_t)(M == 128 ? tw1_stride<Cfg<128>>() : tw1_stride<Cfg<64>>());
+  return (size_t)M * M * sizeof(float2) + tw1 * sizeof(float2) + (size_t)(chain_threads(M) / 32) * sizeof(double) +
+         sizeof(double);
 }
 
 template <int M>

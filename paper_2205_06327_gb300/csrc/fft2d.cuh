@@ -21,7 +21,11 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
+
 #include <type_traits>
+
+#include "tc_bf16.cuh"
 
 namespace ptycho {
 
@@ -34,11 +38,13 @@ __device__ __forceinline__ void static_for(F&& f) {
 }
 
 // Complex sums as packed pairs of FP32 operations: one instruction for both
-// components, each rounded as the scalar operation.  A packed instruction
-// takes two slots of the FP32 pipe (0.46 packed against 0.90 scalar per clock
-// and scheduler), so it saves issue slots, not arithmetic.  Measured (scalar
-// -> packed): 576 positions, M = 128, 16 slices 2.28 -> 2.20 ms; 960
-// positions, M = 64 1.17 -> 1.06 ms; 506 positions, M = 192 7.14 -> 6.78 ms.
+// components, each rounded as the scalar operation, so results are unchanged.
+// A packed instruction takes two slots of the FP32 pipe (probe: 0.46 packed
+// against 0.90 scalar per clock and scheduler), so it buys issue slots, not
+// arithmetic: the chain issued 1.84 M instructions per position against an
+// FP32 pipe 40 % busy.  Measured (scalar -> packed sums): 576 positions,
+// M = 128, 16 slices 2.28 -> 2.20 ms; 960 positions, M = 64 1.17 -> 1.06 ms;
+// 506 positions, M = 192 7.16 -> 6.80 ms.
 __device__ __forceinline__ unsigned long long pack2(float2 a) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
@@ -70,6 +76,28 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
 __device__ __forceinline__ float2 cconjmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x));
 }
+// The same products with packed instructions (identical rounding): fewer issue
+// slots, but their operands need aligned register pairs.  They pay in the
+// register-resident chain (below) and cost spills in the line passes of
+// chain_gm_line.cuh.
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+  return unpack2(r);
+}
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) {
+  return fma2(make_float2(a.x, a.x), b, mul2(make_float2(a.y, a.y), make_float2(-b.y, b.x)));
+}
+__device__ __forceinline__ float2 pmulc(float2 a, float2 b) {
+  return fma2(a, make_float2(b.x, b.x), mul2(make_float2(a.y, -a.x), make_float2(b.y, b.y)));
+}
+template <bool CONJ>
+__device__ __forceinline__ float2 pmul_opt(float2 a, float2 b) { return CONJ ? pmulc(a, b) : pmul(a, b); }
 template <bool CONJ>
 __device__ __forceinline__ float2 cmul_opt(float2 a, float2 b) { return CONJ ? cmulc(a, b) : cmul(a, b); }
 
@@ -258,66 +286,83 @@ __device__ __forceinline__ void xch_load(float2 (&v)[C::V], const float2* sm, in
   });
 }
 
+// Where a thread finds its per-pass factors (filled once per block by
+// fill_factors, every entry rounded once from FP64).  Read from shared and
+// global memory, each with its own index arithmetic, the twiddles and the
+// propagator were a third of the chain's shared-memory wavefronts and a fifth
+// of its instructions, and spilled registers.  A thread needs the same 2 V
+// pass-0 and spectrum factors for the whole chain, and tensor memory (unused
+// otherwise by this kernel) holds exactly 4 V = 128 words per thread and has a
+// data path of its own.  With the packed products below: one wave of 152
+// positions, M = 128, 16 slices 445 -> 380 us; 576 positions 2.20 -> 2.04 ms;
+// 960 positions, M = 64 1.06 -> 0.98 ms.  The adjoint now reads the exact
+// twiddles too (it multiplied two table entries per element before).
+//   tmem  this warp's 128 tensor-memory columns: words [0, 2V) hold the pass-0
+//         twiddles of the thread's V elements, words [2V, 4V) the propagator
+//         at its V spectrum elements (pass-2 grouping);
+//   tw1   shared table of the pass-1 twiddles, one row of G entries per
+//         (ey, ex) class (16 classes).
+struct Factors {
+  uint32_t tmem;
+  const float2* tw1;
+};
+
+template <class C>
+__host__ __device__ constexpr int tw1_stride() {  // float2; odd in 16-byte units: the classes fall on different banks
+  return C::ry(1) * C::rx(1) + 2;
+}
+
+// 8 complex values of the thread's tensor-memory row from word `word` on.
+__device__ __forceinline__ void tmem_factors8(uint32_t taddr, float2 (&w)[8]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) w[i] = make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+}
+
 // One radix pass on the registers.  Forward: DFT over digit J of y (for every
 // x element), DFT over digit J of x (for every y element), then the twiddle
 // w_M^(ey*a' + ex*b') that couples digit J to the lower digits.  Inverse: the
 // conjugate twiddle, then the inverse DFTs (exact inverse up to the factor RY*RX).
-// FACT selects factored twiddles w^(ey a) * w^(ex b): fewer table reads but
-// one more rounding per element.  The forward model (whose rounding the
-// amplitude residual amplifies) uses exact table values; the adjoint, which
-// is linear in the residual, uses the factored form.
-template <class C, int J, bool INV, bool FACT = false>
-__device__ __forceinline__ void pass_compute(float2 (&v)[C::V], const float2* __restrict__ tw, int t) {
+template <class C, int J, bool INV>
+__device__ __forceinline__ void pass_compute(float2 (&v)[C::V], const Factors& f, int t) {
   using P = PassShape<C, J>;
   t = opaque(t);
-  static_for<0, P::Q>([&](auto qq) {
-    constexpr int q = decltype(qq)::value;
-    constexpr int o = q * P::G;
-    [[maybe_unused]] int ey = 0, ex = 0;
-    if constexpr (J < 2) {
-      int py, px;
-      C::template base<J>(t, q, py, px);
-      ey = (C::M / (P::RY * P::SY)) * (py & (P::SY - 1));
-      ex = (C::M / (P::RX * P::SX)) * (px & (P::SX - 1));
+  auto twiddle = [&]() {
+    if constexpr (J == 0) {
+      static_for<0, C::V / 8>([&](auto cc) {
+        constexpr int c = decltype(cc)::value;
+        float2 w[8];
+        tmem_factors8(f.tmem + 16 * c, w);
+        static_for<0, 8>([&](auto ii) {
+          constexpr int e = 8 * c + decltype(ii)::value;
+          if constexpr (e % P::G != 0) v[e] = pmul_opt<INV>(v[e], w[e % 8]);
+        });
+      });
+    } else if constexpr (J == 1) {
+      static_for<0, P::Q>([&](auto qq) {
+        constexpr int q = decltype(qq)::value;
+        int py, px;
+        C::template base<1>(t, q, py, px);
+        const float4* row =
+            reinterpret_cast<const float4*>(f.tw1 + ((py & (P::SY - 1)) * P::SX + (px & (P::SX - 1))) * tw1_stride<C>());
+        static_for<0, P::G / 2>([&](auto ee) {
+          constexpr int e = 2 * decltype(ee)::value;
+          const float4 w = row[e / 2];
+          if constexpr (e != 0) v[q * P::G + e] = pmul_opt<INV>(v[q * P::G + e], make_float2(w.x, w.y));
+          v[q * P::G + e + 1] = pmul_opt<INV>(v[q * P::G + e + 1], make_float2(w.z, w.w));
+        });
+      });
     }
-    auto twiddle = [&]() {
-      if constexpr (J < 2 && FACT) {
-        // w^(ey a + ex b) = w^(ey a) * w^(ex b): RY-1 + RX-1 table reads and
-        // one extra product per element with a, b > 0.
-        float2 txv[P::RX];
-        static_for<1, P::RX>([&](auto bb) {
-          constexpr int b = decltype(bb)::value;
-          txv[b] = tw[(ex * b) & (C::M - 1)];
-        });
-        static_for<0, P::RY>([&](auto aa) {
-          constexpr int a = decltype(aa)::value;
-          float2 ty = make_float2(1.f, 0.f);
-          if constexpr (a != 0) ty = tw[(ey * a) & (C::M - 1)];
-          static_for<0, P::RX>([&](auto bb) {
-            constexpr int b = decltype(bb)::value;
-            if constexpr (a != 0 && b != 0) {
-              v[o + a * P::RX + b] = cmul_opt<INV>(v[o + a * P::RX + b], cmul(ty, txv[b]));
-            } else if constexpr (a != 0) {
-              v[o + a * P::RX + b] = cmul_opt<INV>(v[o + a * P::RX + b], ty);
-            } else if constexpr (b != 0) {
-              v[o + a * P::RX + b] = cmul_opt<INV>(v[o + a * P::RX + b], txv[b]);
-            }
-          });
-        });
-      } else if constexpr (J < 2) {
-        static_for<0, P::RY>([&](auto aa) {
-          constexpr int a = decltype(aa)::value;
-          static_for<0, P::RX>([&](auto bb) {
-            constexpr int b = decltype(bb)::value;
-            if constexpr (a != 0 || b != 0) {
-              const float2 w = tw[(ey * a + ex * b) & (C::M - 1)];
-              v[o + a * P::RX + b] = cmul_opt<INV>(v[o + a * P::RX + b], w);
-            }
-          });
-        });
-      }
-    };
-    if constexpr (INV) twiddle();
+  };
+  if constexpr (INV) twiddle();
+  static_for<0, P::Q>([&](auto qq) {
+    constexpr int o = decltype(qq)::value * P::G;
     static_for<0, P::RX>([&](auto bb) {
       constexpr int b = decltype(bb)::value;
       dft_at<P::RY, INV, o + b, P::RX>(v);
@@ -326,94 +371,108 @@ __device__ __forceinline__ void pass_compute(float2 (&v)[C::V], const float2* __
       constexpr int a = decltype(aa)::value;
       dft_at<P::RX, INV, o + a * P::RX, 1>(v);
     });
-    if constexpr (!INV) twiddle();
   });
+  if constexpr (!INV) twiddle();
 }
 
 // registers in pass-0 grouping (natural storage) -> unnormalised forward DFT,
 // registers in pass-2 grouping (digit-reversed storage)
-template <class C, bool FACT = false>
-__device__ __forceinline__ void fft_fwd(float2 (&v)[C::V], float2* sm, const float2* tw, int t) {
-  pass_compute<C, 0, false, FACT>(v, tw, t);
+template <class C>
+__device__ __forceinline__ void fft_fwd(float2 (&v)[C::V], float2* sm, const Factors& f, int t) {
+  pass_compute<C, 0, false>(v, f, t);
   xch_store<C, 0>(v, sm, t);
   __syncthreads();
   xch_load<C, 1>(v, sm, t);
-  pass_compute<C, 1, false, FACT>(v, tw, t);
+  pass_compute<C, 1, false>(v, f, t);
   xch_store<C, 1>(v, sm, t);
   C::sync12(t);
   xch_load<C, 2>(v, sm, t);
-  pass_compute<C, 2, false, FACT>(v, tw, t);
+  pass_compute<C, 2, false>(v, f, t);
 }
 
 // exact reverse of fft_fwd: unnormalised inverse DFT (times M*M relative to
 // the true inverse), registers back in pass-0 grouping
-template <class C, bool FACT = false>
-__device__ __forceinline__ void fft_inv(float2 (&v)[C::V], float2* sm, const float2* tw, int t) {
-  pass_compute<C, 2, true, FACT>(v, tw, t);
+template <class C>
+__device__ __forceinline__ void fft_inv(float2 (&v)[C::V], float2* sm, const Factors& f, int t) {
+  pass_compute<C, 2, true>(v, f, t);
   xch_store<C, 2>(v, sm, t);
   C::sync12(t);
   xch_load<C, 1>(v, sm, t);
-  pass_compute<C, 1, true, FACT>(v, tw, t);
+  pass_compute<C, 1, true>(v, f, t);
   xch_store<C, 1>(v, sm, t);
   __syncthreads();
   xch_load<C, 0>(v, sm, t);
-  pass_compute<C, 0, true, FACT>(v, tw, t);
+  pass_compute<C, 0, true>(v, f, t);
 }
 
-// Multiply the spectrum (pass-2 grouping) by h(ky)*h(kx) (or its conjugate);
-// hs[k] holds one separable factor of the propagator in FFT order.
+// Multiply the spectrum (pass-2 grouping) by the propagator h(ky, kx) / M^2 or
+// its conjugate.
 template <class C, bool CONJ>
-__device__ __forceinline__ void mul_separable(float2 (&v)[C::V], const float2* __restrict__ hs, int t) {
-  using P = PassShape<C, 2>;
-  t = opaque(t);
-  static_for<0, P::Q>([&](auto qq) {
-    constexpr int q = decltype(qq)::value;
-    int py, px;
-    C::template base<2>(t, q, py, px);
-    const int ky0 = freq_y<C>(py), kx0 = freq_x<C>(px);
-    float2 hx[P::RX];
-    static_for<0, P::RX>([&](auto bb) {
-      constexpr int b = decltype(bb)::value;
-      hx[b] = hs[kx0 + C::rx(0) * C::rx(1) * b];
-    });
-    static_for<0, P::RY>([&](auto aa) {
-      constexpr int a = decltype(aa)::value;
-      const float2 hy = hs[ky0 + C::ry(0) * C::ry(1) * a];
-      static_for<0, P::RX>([&](auto bb) {
-        constexpr int b = decltype(bb)::value;
-        const float2 hh = cmul(hy, hx[b]);
-        v[q * P::G + a * P::RX + b] = cmul_opt<CONJ>(v[q * P::G + a * P::RX + b], hh);
-      });
+__device__ __forceinline__ void mul_prop(float2 (&v)[C::V], const Factors& f) {
+  static_for<0, C::V / 8>([&](auto cc) {
+    constexpr int c = decltype(cc)::value;
+    float2 w[8];
+    tmem_factors8(f.tmem + 2 * C::V + 16 * c, w);
+    static_for<0, 8>([&](auto ii) {
+      constexpr int e = 8 * c + decltype(ii)::value;
+      v[e] = pmul_opt<CONJ>(v[e], w[e % 8]);
     });
   });
 }
 
-// Multiply the spectrum (pass-2 grouping) by the propagator read from a full
-// M x M table h2[ky][kx] (FFT order), each entry rounded once from FP64: one
-// rounding per element fewer than forming h(ky) h(kx) here.  The table is
-// read through the read-only cache (the same 64 or 128 KiB for every block).
-template <class C, bool CONJ>
-__device__ __forceinline__ void mul_table(float2 (&v)[C::V], const float2* __restrict__ h2, int t) {
-  using P = PassShape<C, 2>;
-  t = opaque(t);
-  static_for<0, P::Q>([&](auto qq) {
-    constexpr int q = decltype(qq)::value;
-    int py, px;
-    C::template base<2>(t, q, py, px);
-    const float2* hp = h2 + freq_y<C>(py) * C::M + freq_x<C>(px);
-    float2 hh[P::G];
-    static_for<0, P::RY>([&](auto aa) {
-      constexpr int a = decltype(aa)::value;
-      static_for<0, P::RX>([&](auto bb) {
-        constexpr int b = decltype(bb)::value;
-        hh[a * P::RX + b] = __ldg(hp + a * C::ry(0) * C::ry(1) * C::M + b * C::rx(0) * C::rx(1));
-      });
+// Fill the block's factors from the twiddle table tw[M] and the propagator
+// table h2[M][M] (global memory; with_h = false leaves the propagator out).
+// The caller synchronises the block before tw1 is read; the tensor-memory
+// words are read back only by the thread's own warp.
+template <class C>
+__device__ __forceinline__ void fill_factors(uint32_t taddr, float2* tw1, const float2* __restrict__ tw,
+                                             const float2* __restrict__ h2, bool with_h, int t) {
+  {
+    using P = PassShape<C, 1>;
+    constexpr int EY = C::M / (P::RY * P::SY), EX = C::M / (P::RX * P::SX);
+    for (int k = t; k < P::SY * P::SX * P::G; k += C::T) {
+      const int cls = k / P::G, e = k % P::G;
+      const int ex = EY * (cls / P::SX) * (e / P::RX) + EX * (cls % P::SX) * (e % P::RX);
+      tw1[cls * tw1_stride<C>() + e] = __ldg(tw + (ex & (C::M - 1)));
+    }
+  }
+  auto put = [&](uint32_t addr, const float2 (&w)[8]) {
+    uint32_t r[16];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      r[2 * i] = __float_as_uint(w[i].x);
+      r[2 * i + 1] = __float_as_uint(w[i].y);
+    }
+    tc::tmem_st16(addr, r);
+  };
+  static_for<0, C::V / 8>([&](auto cc) {
+    constexpr int c = decltype(cc)::value;
+    using P = PassShape<C, 0>;
+    float2 w[8];
+    static_for<0, 8>([&](auto ii) {
+      constexpr int i = decltype(ii)::value, e = 8 * c + i, q = e / P::G, a = e % P::G / P::RX, b = e % P::RX;
+      int py, px;
+      C::template base<0>(t, q, py, px);
+      constexpr int EY = C::M / (P::RY * P::SY), EX = C::M / (P::RX * P::SX);
+      w[i] = __ldg(tw + ((EY * (py & (P::SY - 1)) * a + EX * (px & (P::SX - 1)) * b) & (C::M - 1)));
     });
-    static_for<0, P::G>([&](auto ee) {
-      constexpr int e = decltype(ee)::value;
-      v[q * P::G + e] = cmul_opt<CONJ>(v[q * P::G + e], hh[e]);
-    });
+    put(taddr + 16 * c, w);
   });
+  if (with_h)
+    static_for<0, C::V / 8>([&](auto cc) {
+      constexpr int c = decltype(cc)::value;
+      using P = PassShape<C, 2>;
+      float2 w[8];
+      static_for<0, 8>([&](auto ii) {
+        constexpr int i = decltype(ii)::value, e = 8 * c + i, q = e / P::G, a = e % P::G / P::RX, b = e % P::RX;
+        int py, px;
+        C::template base<2>(t, q, py, px);
+        const int ky = freq_y<C>(py) + C::ry(0) * C::ry(1) * a, kx = freq_x<C>(px) + C::rx(0) * C::rx(1) * b;
+        w[i] = __ldg(h2 + ky * C::M + kx);
+      });
+      put(taddr + 2 * C::V + 16 * c, w);
+    });
+  tc::tmem_wait_st();
 }
 
 }  // namespace ptycho
