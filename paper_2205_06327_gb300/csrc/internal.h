@@ -40,7 +40,7 @@ struct ChainArgs {
                           // patches | 1 parked adjoint state][ws_n][M][M]
   float2* ws_gphi;        // GRAD: [S][ws_n][M][M] gradient w.r.t. each slice's exit wave
   float2* ws_gp;          // [ws_n][M][M]      per-position probe gradient
-  double* loss_part;      // [n_pos]
+  double* loss_part;      // [n_pos] (generic windows: [n_pos][gm_loss_parts(M)])
   float2* psi_out;        // [N][M][M] or null (forward mode)
   float* int_out;         // [N][M][M] or null (forward mode)
   int* status;            // device error word (PTYCHO_ERR_POSITION on a bad window)
@@ -74,12 +74,8 @@ cudaError_t launch_chain_tc(ChainMode mode, const ChainArgs& a, const uint32_t* 
                             cudaStream_t st);
 
 // chain_gm.cu (any window M = 2^a 3^b, 8 <= M <= 4096, FP32)
-struct GmPlan {
-  int n;      // radix stages
-  int r[16];  // radices (4, 2, 3)
-};
-bool gm_supported(int M, GmPlan* plan);
-size_t gm_fft_smem_bytes(int M);
+bool gm_supported(int M);
+int gm_loss_parts(int M);  // loss parts the chain writes per position
 cudaError_t gm_prepare(int M);
 cudaError_t launch_chain_gm(ChainMode mode, const ChainArgs& a, float2* wv, int M, int* n_launches,
                             cudaStream_t st);

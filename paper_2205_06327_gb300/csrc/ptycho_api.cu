@@ -185,7 +185,8 @@ struct ptycho_plan_s {
   float2* ws_gp = nullptr;    // [chunk][M][M]
   float2* wv = nullptr;       // generic-window path: [chunk][M][M] waves of the chunk
   float2* gp_part = nullptr;  // [kProbeSplit][M][M]
-  double* loss_part = nullptr;  // [chunk]
+  double* loss_part = nullptr;  // [chunk][loss_parts]
+  int loss_parts = 1;           // loss parts per position (generic-window path: its line blocks)
   double* d_scal = nullptr;   // [8]: 0 loss, 1 |gO|^2, 2 |gP|^2, 3 trial loss
   double* norm_part = nullptr;  // [kNormParts]
   int* d_status = nullptr;
@@ -281,7 +282,7 @@ int dev_alloc(T** p, size_t count, const char* what) {
 bool fused_window(int M) { return M == 64 || M == 128; }
 
 int validate_params(const ptycho_params& p) {
-  if (!fused_window(p.M) && !(p.precision == PTYCHO_FP32 && gm_supported(p.M, nullptr)))
+  if (!fused_window(p.M) && !(p.precision == PTYCHO_FP32 && gm_supported(p.M)))
     return fail(PTYCHO_ERR_UNSUPPORTED,
                 "probe window M must be 64 or 128, or (FP32) a product of powers of 2 and 3 in [8, 4096]");
   if (p.S < 1) return fail(PTYCHO_ERR_ARG, "S must be >= 1");
@@ -463,7 +464,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
     r.ws_psi = pl->ws_psi + (size_t)off * MM;
     r.ws_gphi = pl->ws_gphi ? pl->ws_gphi + (size_t)off * MM : nullptr;
     r.ws_gp = pl->ws_gp + (size_t)off * MM;
-    r.loss_part = pl->loss_part + off;
+    r.loss_part = pl->loss_part + (size_t)off * pl->loss_parts;
     return r;
   };
   auto launch_chain_for = [&](const ChainArgs& ca) -> int {
@@ -573,7 +574,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
     }
     if (grad_probe)
       TIMED(K_PROBE, 2, launch_probe_grad(pl->ws_gp, n, p.M, pl->gp_part, kProbeSplit, grad_probe, ci > 0, st));
-    TIMED(K_OTHER, 1, launch_loss_accum(pl->loss_part, n, pl->d_scal + slot, ci > 0, st));
+    TIMED(K_OTHER, 1, launch_loss_accum(pl->loss_part, n * pl->loss_parts, pl->d_scal + slot, ci > 0, st));
   }
   return PTYCHO_OK;
 }
@@ -687,6 +688,7 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
     if (chunk > blocks_per_wave) chunk -= chunk % blocks_per_wave;
   }
   pl->chunk = (int)chunk;
+  if (gm) pl->loss_parts = gm_loss_parts(M);
   // Chain blocks resident on the GPU at once: the occupancy of the FP32
   // gradient kernel, or one split-product block per SM (all of tensor memory).
   if (!gm) pl->wave = pl->sm_count * (p.precision == PTYCHO_FP32 ? chain_blocks_per_sm(M) : 1);
@@ -700,7 +702,7 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
   if (!rc) rc = dev_alloc(&pl->ws_gp, (size_t)pl->chunk * MM, "probe-gradient workspace");
   if (!rc && gm) rc = dev_alloc(&pl->wv, (size_t)pl->chunk * MM, "generic-window wave buffer");
   if (!rc) rc = dev_alloc(&pl->gp_part, (size_t)kProbeSplit * MM, "probe-gradient partials");
-  if (!rc) rc = dev_alloc(&pl->loss_part, (size_t)pl->chunk, "loss partials");
+  if (!rc) rc = dev_alloc(&pl->loss_part, (size_t)pl->chunk * pl->loss_parts, "loss partials");
   if (!rc) rc = dev_alloc(&pl->d_scal, 8, "scalars");
   if (!rc) rc = dev_alloc(&pl->norm_part, kNormParts, "norm partials");
   if (!rc) rc = dev_alloc(&pl->d_status, 1, "status");
