@@ -115,8 +115,12 @@ typedef struct {
   int64_t workspace_bytes; /* cap on the plan's workspace; 0 = 8 GiB.  Positions
                               are processed in chunks that fit the cap, so the
                               memory used does not grow with N. */
-  int32_t tile_h, tile_w;  /* object-gradient accumulation tile (pixels);
-                              0 = 32 x 32.  tile_h * tile_w <= 8192. */
+  int32_t tile_h, tile_w;  /* object-gradient accumulation tile (pixels), 0 = the
+                              library's choice.  tile_h * tile_w <= 8192 (a
+                              side left 0 counts 32).  Rows are taken 8 at a
+                              time whatever tile_h; tile_w columns, but at
+                              least a window's and at most 1024.  The shape
+                              changes the speed only. */
   int32_t ckpt_every; /* 0: keep every slice's wave for the adjoint (fastest).
                          L >= 1: per-slice recomputation.  Keep the waves
                          entering every L-th slice (checkpoints), and during

@@ -16,7 +16,7 @@ import torch
 
 from .api import Geometry, Plan
 
-CANDIDATES = ((16, 16), (32, 32), (32, 64), (64, 32), (64, 64), (16, 64))
+CANDIDATES = ((0, 0), (8, 128), (8, 192), (8, 256), (8, 384), (8, 512))  # (0, 0): the library's choice
 
 
 def cache_path() -> str:
@@ -42,7 +42,7 @@ def _save(d: dict) -> None:
 
 
 def key_for(geom: Geometry, precision: str, ckpt_every: int = 0) -> str:
-    return f"M{geom.M}_S{geom.S}_H{geom.H}_W{geom.W}_N{geom.N}_{precision}" + (f"_rc{ckpt_every}" if ckpt_every else "")
+    return f"bands_M{geom.M}_S{geom.S}_H{geom.H}_W{geom.W}_N{geom.N}_{precision}" + (f"_rc{ckpt_every}" if ckpt_every else "")
 
 
 def tune_tile(geom: Geometry, pos, probe, obj, meas, device, precision: str = "fp32",

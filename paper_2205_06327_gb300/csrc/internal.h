@@ -81,12 +81,13 @@ cudaError_t launch_chain_gm(ChainMode mode, const ChainArgs& a, float2* wv, int 
                             cudaStream_t st);
 
 // reduce_kernels.cu
-constexpr int kDefaultTile = 32;  // default owner tile of the object-gradient accumulation
+constexpr int kDefaultTile = 32;  // stands for the other side of a plan's tile given one, in the size check
 struct AccumArgs {
   const int2* pos;
   int pos_begin, n_pos;
   int M, S, H, W;
-  int tile_h, tile_w;
+  int tile_w;               // tile columns asked for (0: chosen by the launch)
+  int seg_w;                // set by the launch: tile columns a warp holds in flight at most
   const float2* probe;      // wave entering slice 0 (= probe)
   int ws_n;                 // slice stride (positions) of ws_psi / ws_gphi
   const float2* ws_psi;     // [S-1][ws_n][M][M]

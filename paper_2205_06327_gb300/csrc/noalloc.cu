@@ -207,8 +207,7 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
       g.S = p.S;
       g.H = p.H;
       g.W = p.W;
-      g.tile_h = th;
-      g.tile_w = tw_;
+      g.tile_w = p.tile_w;
       g.probe = a.probe;
       g.ws_n = chunk;
       g.ws_psi = ws_psi;

@@ -421,8 +421,7 @@ int accum_part(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, floa
   g.S = p.S;
   g.H = p.H;
   g.W = p.W;
-  g.tile_h = p.tile_h ? p.tile_h : kDefaultTile;
-  g.tile_w = p.tile_w ? p.tile_w : kDefaultTile;
+  g.tile_w = p.tile_w;
   g.probe = reinterpret_cast<const float2*>(probe);
   g.ws_n = pl->chunk;
   g.ws_psi = pl->ws_psi + (size_t)off * MM;
@@ -497,8 +496,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
     g.S = p.S;
     g.H = p.H;
     g.W = p.W;
-    g.tile_h = p.tile_h ? p.tile_h : kDefaultTile;
-    g.tile_w = p.tile_w ? p.tile_w : kDefaultTile;
+    g.tile_w = p.tile_w;
     g.probe = a.probe;
     g.ws_n = pl->chunk;
     g.ws_psi = pl->ws_psi + (size_t)off * MM;

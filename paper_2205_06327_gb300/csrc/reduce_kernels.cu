@@ -7,7 +7,7 @@
 // sum_i conj(psi_{i,s}) * g_phi_{i,s} placed at window i.  The object is
 // tessellated into tiles; one block owns one (tile, slice), walks the
 // positions whose window meets its tile in ascending order and sums their
-// contributions in registers.  Every output pixel therefore has exactly one
+// contributions on chip.  Every output pixel therefore has exactly one
 // writer and a fixed summation order: no atomics, bit-reproducible.
 #include "internal.h"
 #include "../../include/ptycho.h"
@@ -16,150 +16,203 @@ namespace ptycho {
 
 namespace {
 
-__device__ __forceinline__ float2 ld_stream(const float2* p) { return __ldcs(p); }
-
 constexpr int kAccThreads = 256;
+constexpr int kAccWarps = kAccThreads / 32;
+constexpr int kAccDefaultCols = 512;
+constexpr int kAccMaxCols = 1024;
+constexpr int kAccBatch = 4 * kAccThreads;  // positions listed at a time
 
-// Accumulation shape: positions whose loads are in flight together, and
-// resident blocks per SM the kernel is compiled for.
-#ifndef PTYCHO_ACC_UNROLL
-#define PTYCHO_ACC_UNROLL 4
-#endif
-#ifndef PTYCHO_ACC_MIN_BLOCKS
-#define PTYCHO_ACC_MIN_BLOCKS 2
-#endif
-constexpr int kAccUnroll = PTYCHO_ACC_UNROLL;
-constexpr int kAccPPT = 4;     // pixels per thread per pixel group
+template <int VEC>
+struct AccVec;
+template <>
+struct AccVec<2> {
+  using type = float4;
+  static __device__ __forceinline__ float4 zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+  static __device__ __forceinline__ float2 get(const float4& v, int i) {
+    return i ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+  }
+};
+template <>
+struct AccVec<1> {
+  using type = float2;
+  static __device__ __forceinline__ float2 zero() { return make_float2(0.f, 0.f); }
+  static __device__ __forceinline__ float2 get(const float2& v, int) { return v; }
+};
 
-// One block owns one (tile, slice).  The tile's pixels are processed in
-// groups of kAccPPT * 256; for each group the block walks the positions whose
-// window meets the group's rows, in ascending order.
-__global__ void __launch_bounds__(kAccThreads, PTYCHO_ACC_MIN_BLOCKS) k_accum_obj_grad(const AccumArgs a) {
-  __shared__ int2 lpos[kAccThreads];
-  __shared__ int lidx[kAccThreads];
-  __shared__ int wcount[kAccThreads / 32];
+// One block owns one (tile, slice) and each of its 8 warps one row of the
+// tile: the row's sums live in shared memory and only that warp touches them.
+// The warp walks the positions whose window covers its row in ascending order
+// and streams that window row of psi and g_phi, VEC pixels per lane and step
+// (16-byte loads for even windows), K steps per position, with the loads of U
+// positions in flight before the first is added.
+//
+// The kernel is bound by HBM: it reads the two workspace arrays once.  With
+// threads tied to the pixels of a 32 x 32 tile, a third of the loads fell
+// outside the window and the rest came in 256-byte pieces of rows 1 KB apart.
+// Here lanes follow the window, so a full row keeps every lane busy, and
+// neighbouring warps read neighbouring rows of the same windows.  Measured
+// (tile 32 x 32 -> bands): 576 positions, M = 128, 16 slices 876 -> 620 us (both
+// parts, one beside the chain's last wave); 225 positions, M = 192, 12 slices
+// 362 -> 238 us (6.7 TB/s); 930 positions, M = 96 499 -> 338 us; finished
+// patches of 3600 positions, M = 128, 30 slices 4.72 -> 3.43 ms.  Fewer loads
+// in flight with more blocks per SM (half of them, 4 blocks) gave 721 / 276 /
+// 451 us; 8 steps instead of 16 for finished patches 4.02 ms.
+// The probe need not be 16-byte aligned (8 bytes are asked of the caller).
+template <int VEC>
+__device__ __forceinline__ typename AccVec<VEC>::type probe_load(const float2* p) {
+  if constexpr (VEC == 2) {
+    const float2 u = __ldg(p), v = __ldg(p + 1);
+    return make_float4(u.x, u.y, v.x, v.y);
+  } else {
+    return __ldg(p);
+  }
+}
+
+template <int K, int VEC, bool PATCH>
+__global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumArgs a) {
+  using V = AccVec<VEC>;
+  using vec = typename V::type;
+  constexpr int STEPS = PATCH ? 16 : 8, U = STEPS / K;
+  __shared__ int2 lpos[kAccBatch];
+  __shared__ int lidx[kAccBatch];
+  __shared__ int wcount[kAccWarps];
+  extern __shared__ float2 acc[];  // [8][tile_w]
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int z = blockIdx.z;  // slice s_begin + z
+  const int z = blockIdx.x % a.n_slices, b = blockIdx.x / a.n_slices;  // slice s_begin + z
   const int s = a.s_begin + z;
   const int M = a.M;
-  const int ty0 = blockIdx.y * a.tile_h, tx0 = blockIdx.x * a.tile_w;
-  const int th = min(a.tile_h, a.H - ty0), tw = min(a.tile_w, a.W - tx0);
-  const int npix = th * tw;
+  // Blocks in launch order: slices, then tile columns, then tile rows from
+  // the middle outwards (the middle rows, which most windows cover, first).
+  const int nc = (a.W + a.tile_w - 1) / a.tile_w, nr = (a.H + kAccWarps - 1) / kAccWarps;
+  const int rank = b / nc;
+  const int ty0 = kAccWarps * (nr / 2 + (rank % 2 ? -(rank + 1) / 2 : rank / 2));
+  const int tx0 = a.tile_w * (b % nc);
+  const int th = min(kAccWarps, a.H - ty0), tw = min(a.tile_w, a.W - tx0);
+  const int y = ty0 + w;                  // this warp's object row (if w < th)
+  float2* arow = acc + w * a.tile_w;
   const size_t MM = (size_t)M * M;
   const float2* gphi_s = a.ws_gphi + (size_t)(a.seg_slots ? z : s) * a.ws_n * MM;
-  const float2* psi_s =
-      s > 0 && !a.patch_mode ? a.ws_psi + (size_t)(a.seg_slots ? z : s - 1) * a.ws_n * MM : nullptr;
-  float2* out = a.grad_obj + (size_t)s * a.H * a.W;
-  constexpr int GROUP = kAccPPT * kAccThreads;
+  const float2* psi_s = s > 0 && !PATCH ? a.ws_psi + (size_t)(a.seg_slots ? z : s - 1) * a.ws_n * MM : nullptr;
+  for (int x = lane; x < tw; x += 32) arow[x] = make_float2(0.f, 0.f);
 
-  for (int pg0 = 0; pg0 < npix; pg0 += GROUP) {
-    // Pixel k of this thread: p = pg0 + t + 256 k in the tile, row-major.
-    int rowk[kAccPPT], colk[kAccPPT];
-    float2 acc[kAccPPT];
+  for (int base = 0; base < a.n_pos; base += kAccBatch) {
+    // Positions of this batch whose window meets the tile, in ascending order
+    // (four consecutive positions per thread, block prefix sum).
+    int2 r[4];
+    unsigned hit = 0;
 #pragma unroll
-    for (int k = 0; k < kAccPPT; ++k) {
-      const int p = pg0 + t + kAccThreads * k;
-      rowk[k] = p < npix ? p / tw : (1 << 28);
-      colk[k] = p < npix ? p % tw : 0;
-      acc[k] = make_float2(0.f, 0.f);
+    for (int k = 0; k < 4; ++k) {
+      const int il = base + 4 * t + k;
+      r[k] = il < a.n_pos ? a.pos[a.pos_begin + il] : make_int2(-1, -1);
+      const bool ok = r[k].x >= 0 && r[k].y >= 0 && r[k].x <= a.H - M && r[k].y <= a.W - M;
+      if (ok && r[k].x < ty0 + th && r[k].x + M > ty0 && r[k].y < tx0 + tw && r[k].y + M > tx0) hit |= 1u << k;
     }
-    const int gy0 = ty0 + pg0 / tw;
-    const int gy1 = ty0 + min(npix - 1, pg0 + GROUP - 1) / tw + 1;  // rows [gy0, gy1)
+    const int n = __popc(hit);
+    int off = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, off, d);
+      if (lane >= d) off += v;
+    }
+    __syncthreads();  // the previous batch's list is read
+    if (lane == 31) wcount[w] = off;
+    __syncthreads();
+    int slot = off - n, total = 0;
+#pragma unroll
+    for (int k = 0; k < kAccWarps; ++k) {
+      slot += k < w ? wcount[k] : 0;
+      total += wcount[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (hit >> k & 1) {
+        lpos[slot] = r[k];
+        lidx[slot++] = base + 4 * t + k;
+      }
+    __syncthreads();
 
-    for (int base = 0; base < a.n_pos; base += kAccThreads) {
-      // Positions of this batch whose window meets the group, compacted in
-      // ascending order (ballot + warp prefix): the summation order.
-      const int il = base + t;
-      bool hit = false;
-      int2 r = make_int2(0, 0);
-      if (il < a.n_pos) {
-        r = a.pos[a.pos_begin + il];
-        const bool ok = r.x >= 0 && r.y >= 0 && r.x <= a.H - M && r.y <= a.W - M;
-        hit = ok && r.x < gy1 && r.x + M > gy0 && r.y < tx0 + tw && r.y + M > tx0;
-      }
-      const unsigned b = __ballot_sync(0xffffffffu, hit);
-      if (lane == 0) wcount[w] = __popc(b);
-      __syncthreads();
-      int off = 0, total = 0;
+    if (w >= th) continue;
+    for (int sx0 = 0; sx0 < tw; sx0 += a.seg_w) {
+      const int sx1 = min(tw, sx0 + a.seg_w);
+      for (int j0 = 0; j0 < total; j0 += 32) {
+        int2 rj = make_int2(0, 0);
+        int ij = 0;
+        bool in = false;
+        if (j0 + lane < total) {
+          rj = lpos[j0 + lane];
+          ij = lidx[j0 + lane];
+          in = rj.x <= y && y < rj.x + M && rj.y - tx0 < sx1 && rj.y - tx0 + M > sx0;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, in);
+        while (todo) {
+          // The loads of up to U positions, then their sums in order.
+          vec pv[U][K], gv[U][K];
+          int cx[U], lo[U], hi[U];  // tile column of window column 0; window columns [lo, hi) of the segment
 #pragma unroll
-      for (int k = 0; k < kAccThreads / 32; ++k) {
-        off += k < w ? wcount[k] : 0;
-        total += wcount[k];
-      }
-      if (hit) {
-        const int slot = off + __popc(b & ((1u << lane) - 1u));
-        lpos[slot] = r;
-        lidx[slot] = il;
-      }
-      __syncthreads();
-      for (int j0 = 0; j0 < total; j0 += kAccUnroll) {
-        // Issue the loads of up to kAccUnroll positions, then add them in
-        // order.  Pixels outside a window load zeros, whose product adds
-        // exactly nothing.
-        float2 pv[kAccUnroll][kAccPPT], gv[kAccUnroll][kAccPPT];
+          for (int u = 0; u < U; ++u) {
+            const bool live = todo != 0;
+            const int src = live ? __ffs(todo) - 1 : 0;
+            todo &= todo - 1;
+            const int ry = __shfl_sync(0xffffffffu, rj.x, src), rx = __shfl_sync(0xffffffffu, rj.y, src);
+            const int i = __shfl_sync(0xffffffffu, ij, src);
+            cx[u] = rx - tx0;
+            lo[u] = max(0, sx0 - cx[u]);
+            hi[u] = live ? min(M, sx1 - cx[u]) : 0;
+            const size_t row_off = (size_t)i * MM + (size_t)(y - ry) * M;
+            const float2* gp = gphi_s + row_off;
+            const float2* pp = PATCH ? nullptr : s > 0 ? psi_s + row_off : a.probe + (size_t)(y - ry) * M;
+            const int x0 = (lo[u] & ~(VEC - 1)) + VEC * lane;
 #pragma unroll
-        for (int u = 0; u < kAccUnroll; ++u) {
-          const int j = j0 + u;
-          const bool live = j < total;
-          const int2 rr = lpos[live ? j : 0];
-          const int i = lidx[live ? j : 0];
-          const int oy0 = ty0 - rr.x, ox0 = tx0 - rr.y;
-          const float2* gp = gphi_s + (size_t)i * MM;
-          const float2* pp = s > 0 && !a.patch_mode ? psi_s + (size_t)i * MM : a.probe;
-          if (a.patch_mode) {  // finished patches conj(psi) g_phi
-#pragma unroll
-            for (int k = 0; k < kAccPPT; ++k) {
-              const int oy = oy0 + rowk[k], ox = ox0 + colk[k];
-              const bool in = live && (unsigned)oy < (unsigned)M && (unsigned)ox < (unsigned)M;
-              pv[u][k] = in ? ld_stream(gp + oy * M + ox) : make_float2(0.f, 0.f);
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < kAccPPT; ++k) {
-              const int oy = oy0 + rowk[k], ox = ox0 + colk[k];
-              const bool in = live && (unsigned)oy < (unsigned)M && (unsigned)ox < (unsigned)M;
-              const int idx = in ? oy * M + ox : 0;
-              pv[u][k] = in ? (s > 0 ? ld_stream(pp + idx) : __ldg(pp + idx)) : make_float2(0.f, 0.f);
-              gv[u][k] = in ? ld_stream(gp + idx) : make_float2(0.f, 0.f);
+            for (int k = 0; k < K; ++k) {
+              const int x = x0 + 32 * VEC * k;
+              const bool ld = x < hi[u];
+              gv[u][k] = ld ? __ldcs(reinterpret_cast<const vec*>(gp + x)) : V::zero();
+              if constexpr (!PATCH)
+                pv[u][k] = !ld ? V::zero()
+                               : s > 0 ? __ldcs(reinterpret_cast<const vec*>(pp + x)) : probe_load<VEC>(pp + x);
             }
           }
-        }
-        if (a.patch_mode) {
 #pragma unroll
-          for (int u = 0; u < kAccUnroll; ++u) {
+          for (int u = 0; u < U; ++u) {
+            const int x0 = (lo[u] & ~(VEC - 1)) + VEC * lane;
 #pragma unroll
-            for (int k = 0; k < kAccPPT; ++k) {
-              acc[k].x += pv[u][k].x;
-              acc[k].y += pv[u][k].y;
+            for (int k = 0; k < K; ++k) {
+#pragma unroll
+              for (int e = 0; e < VEC; ++e) {
+                const int x = x0 + 32 * VEC * k + e;
+                if (x >= lo[u] && x < hi[u]) {
+                  float2* o = arow + cx[u] + x;
+                  float2 v = *o;
+                  const float2 g = V::get(gv[u][k], e);
+                  if constexpr (PATCH) {  // finished patches conj(psi) g_phi
+                    v.x += g.x;
+                    v.y += g.y;
+                  } else {
+                    const float2 p = V::get(pv[u][k], e);
+                    v.x = fmaf(p.x, g.x, fmaf(p.y, g.y, v.x));
+                    v.y = fmaf(p.x, g.y, fmaf(-p.y, g.x, v.y));
+                  }
+                  *o = v;
+                }
+              }
             }
-          }
-        } else {
-#pragma unroll
-          for (int u = 0; u < kAccUnroll; ++u) {
-#pragma unroll
-            for (int k = 0; k < kAccPPT; ++k) {
-              const float2 p = pv[u][k], g = gv[u][k];
-              acc[k].x = fmaf(p.x, g.x, fmaf(p.y, g.y, acc[k].x));
-              acc[k].y = fmaf(p.x, g.y, fmaf(-p.y, g.x, acc[k].y));
-            }
+            __syncwarp();  // the next position's lanes fall on other columns
           }
         }
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int k = 0; k < kAccPPT; ++k) {
-      if (rowk[k] < th) {
-        float2* o = out + (size_t)(ty0 + rowk[k]) * a.W + (tx0 + colk[k]);
-        float2 val = acc[k];
-        if (a.accumulate) {
-          const float2 prev = *o;
-          val.x += prev.x;
-          val.y += prev.y;
-        }
-        *o = val;
       }
     }
+  }
+  __syncwarp();
+  if (w >= th) return;
+  float2* out = a.grad_obj + (size_t)s * a.H * a.W + (size_t)y * a.W + tx0;
+  for (int x = lane; x < tw; x += 32) {
+    float2 val = arow[x];
+    if (a.accumulate) {
+      const float2 prev = out[x];
+      val.x += prev.x;
+      val.y += prev.y;
+    }
+    out[x] = val;
   }
 }
 
@@ -261,12 +314,65 @@ __global__ void k_check_positions(const int2* __restrict__ pos, int n, int M, in
 
 }  // namespace
 
-cudaError_t launch_accum_obj_grad(const AccumArgs& a, cudaStream_t st) {
+namespace {
+
+template <int K, int VEC>
+cudaError_t accum_launch(const AccumArgs& a, dim3 grid, cudaStream_t st) {
+  const size_t smem = (size_t)kAccWarps * a.tile_w * sizeof(float2);
+  const auto k = a.patch_mode ? k_accum_obj_grad<K, VEC, true> : k_accum_obj_grad<K, VEC, false>;
+  if (smem > kAccDefaultCols * kAccWarps * sizeof(float2)) {  // beyond the 48 KB every kernel may use
+    const cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kAccMaxCols * kAccWarps * (int)sizeof(float2));
+    if (e != cudaSuccess) return e;
+  }
+  k<<<grid, kAccThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <int VEC>
+cudaError_t accum_steps(int steps, const AccumArgs& a, dim3 grid, cudaStream_t st) {
+  switch (steps) {
+    case 1: return accum_launch<1, VEC>(a, grid, st);
+    case 2: return accum_launch<2, VEC>(a, grid, st);
+    case 3: return accum_launch<3, VEC>(a, grid, st);
+    case 4: return accum_launch<4, VEC>(a, grid, st);
+    default: return accum_launch<8, VEC>(a, grid, st);
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_accum_obj_grad(const AccumArgs& args, cudaStream_t st) {
+  AccumArgs a = args;
   const int ns = a.n_slices > 0 ? a.n_slices : a.S - a.s_begin;
   if (a.s_begin < 0 || ns <= 0 || a.s_begin + ns > a.S) return cudaErrorInvalidValue;
-  const dim3 grid((a.W + a.tile_w - 1) / a.tile_w, (a.H + a.tile_h - 1) / a.tile_h, ns);
-  k_accum_obj_grad<<<grid, kAccThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  // Tiles are bands of 8 rows (one per warp).  Their columns: the whole width
+  // (up to kAccDefaultCols), halved while that leaves fewer than three blocks
+  // per SM and still covers a window; a plan's tile may ask for other columns,
+  // at least a window's.  (Halving measured: 230 blocks 4.73 -> 3.43 ms for the
+  // patches above, 385 blocks at M = 96 374 -> 338 us; 552 blocks at M = 192 238
+  // -> 284 us.)
+  if (a.tile_w == 0) {
+    const int n = (a.W + kAccDefaultCols - 1) / kAccDefaultCols;
+    a.tile_w = (a.W + n - 1) / n;
+    auto blocks = [&]() { return (int64_t)ns * ((a.H + kAccWarps - 1) / kAccWarps) * ((a.W + a.tile_w - 1) / a.tile_w); };
+    while (blocks() < 456 && (a.tile_w + 1) / 2 >= a.M) a.tile_w = (a.tile_w + 1) / 2;
+  } else {
+    const int least = a.M < a.W ? a.M : a.W;
+    if (a.tile_w < least) a.tile_w = least;
+    if (a.tile_w > kAccMaxCols) a.tile_w = kAccMaxCols;
+  }
+  // Window rows start on 16 bytes for even M (the workspace is aligned).
+  const int vec = a.M % 2 == 0 ? 2 : 1, step = 32 * vec;
+  a.seg_w = a.tile_w;
+  if (a.M > 8 * step && a.tile_w + vec - 1 > 8 * step) a.seg_w = 8 * step - vec + 1;
+  const int span = a.seg_w + vec - 1 < a.M ? a.seg_w + vec - 1 : a.M;
+  const int steps = (span + step - 1) / step;
+  a.n_slices = ns;
+  const int64_t blocks = (int64_t)ns * ((a.W + a.tile_w - 1) / a.tile_w) * ((a.H + kAccWarps - 1) / kAccWarps);
+  if (blocks > INT32_MAX) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)blocks);
+  return vec == 2 ? accum_steps<2>(steps, a, grid, st) : accum_steps<1>(steps, a, grid, st);
 }
 
 cudaError_t launch_probe_grad(const float2* ws_gp, int n_pos, int M, float2* part, int n_split,
