@@ -41,6 +41,7 @@ struct GmPass {
 // Launches of one window's instance.
 struct GmInstance {
   int M;
+  int r1, r2, r3;
   int parts;  // loss parts per position (blocks of the residual pass)
   cudaError_t (*prepare)();
   cudaError_t (*launch)(GmKind kind, const ChainArgs& a, const GmPass& g, cudaStream_t st);
@@ -297,13 +298,19 @@ __device__ __forceinline__ void gm_skip(const GmBlock& b, int L, int parts, int 
 // inverts the R1 digit into the same registers phase A loaded.  A two-factor
 // propagation so costs two shared-memory round trips per element (Stockham
 // stages of radix 8/8/3 cost five) and the last phase of one propagation, the
-// transmission and the first phase of the next run in registers.
+// transmission and the first phase of the next run in registers.  ncu on 225
+// positions at M = 192 (4 blocks of 256 threads, 64 registers): the shared
+// pipe 60-67 %, FP32 37-39 %, issue 45 %, the largest stall the block barrier,
+// then global loads.  So the shapes below take small blocks (96-128 threads,
+// several items each, many blocks per SM to cover the barriers) and registers
+// enough not to spill.
 //
 // Slots: rows keep line li's element (k1, k2, j2) at li LS + k1 PK + k2 PJ + j2
 // with PJ odd and PK = 16/R1 modulo 16 for R1 | 16, so that the 16 lanes of a
 // half-warp fall on different 8-byte banks in every phase; columns
-// interleave the block's lines ((k1, k2, j2) L + li), so consecutive lanes
-// take consecutive columns, in shared and in global memory.
+// interleave the block's lines ((k1 PK + k2 PJ + j2) L + li), so consecutive
+// lanes take consecutive columns, in shared and in global memory; with fewer
+// than 16 lines PJ and PK are odd, for the same reason.
 // ---------------------------------------------------------------------------
 constexpr int gm_pk(int R1, int R2, int PJ) {
   int p = R2 * PJ;
@@ -322,7 +329,11 @@ struct GmShape {
   static constexpr int PT = R3 | 1;  // pitch of the phase-C twiddle rows
   static constexpr int TA = R2 == 1 ? R1 * PT : M, TB = R2 == 1 ? 0 : R2 * PT;
   static_assert(M % L == 0 && T % 32 == 0, "whole lines per block, whole warps");
-  static constexpr int line_slots(bool cols) { return cols ? M : R1 * gm_pk(R1, R2, R3 | 1); }
+  static constexpr int pj(bool cols) { return cols && L % 16 == 0 ? R3 : R3 | 1; }
+  static constexpr int pk(bool cols) {
+    return !cols ? gm_pk(R1, R2, pj(false)) : R2 == 1 ? pj(true) : L % 16 == 0 ? R2 * R3 : (R2 * pj(true)) | 1;
+  }
+  static constexpr int line_slots(bool cols) { return R1 * pk(cols); }
   static constexpr size_t smem(bool cols) {
     return ((size_t)L * line_slots(cols) + TA + TB + M) * sizeof(float2) + (T / 32) * sizeof(double);
   }
@@ -331,7 +342,7 @@ struct GmShape {
 template <class P, bool COLS>
 struct GmLines {
   static constexpr int R1 = P::R1, R2 = P::R2, R3 = P::R3, L = P::L, T = P::T, MI = P::MI;
-  static constexpr int PJ = COLS ? R3 : (R3 | 1), PK = COLS ? R2 * R3 : gm_pk(R1, R2, R3 | 1), LS = R1 * PK;
+  static constexpr int PJ = P::pj(COLS), PK = P::pk(COLS), LS = R1 * PK;
   float2* D;         // the block's lines
   const float2* TA;  // w_M^(k1 j): [R1][PT] (two factors) or [R1][M/R1]
   const float2* TB;  // w_(M/R1)^(k2 j2): [R2][PT] (three factors)
@@ -574,7 +585,7 @@ cudaError_t gm_launch_ct(GmKind kind, const ChainArgs& a, const GmPass& g, cudaS
 
 template <class P>
 constexpr GmInstance gm_instance() {
-  return GmInstance{P::M, P::M / P::L, gm_prepare_ct<P>, gm_launch_ct<P>};
+  return GmInstance{P::M, P::R1, P::R2, P::R3, P::M / P::L, gm_prepare_ct<P>, gm_launch_ct<P>};
 }
 
 }  // namespace

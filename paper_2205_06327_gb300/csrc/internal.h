@@ -31,6 +31,7 @@ struct ChainArgs {
   int S, H, W;
   const float2* tw;       // [M]   w_M^e = exp(-2 pi i e / M)
   const float2* hs;       // [M]   one separable factor of the propagator, times 1/M
+                          // (generic windows: divided by gm_factor_gain)
   const float2* h2;       // [M][M] the propagator h(ky) h(kx) / M^2 (register-resident kernels)
   int ws_n;               // positions the workspace holds (slice stride of ws_psi / ws_gphi)
   int ckpt_L;             // recompute mode: checkpoint every ckpt_L slices
@@ -75,6 +76,7 @@ cudaError_t launch_chain_tc(ChainMode mode, const ChainArgs& a, const uint32_t* 
 
 // chain_gm.cu (any window M = 2^a 3^b, 8 <= M <= 4096, FP32)
 bool gm_supported(int M);
+void gm_factor_gain(int M, double* gain);
 int gm_loss_parts(int M);  // loss parts the chain writes per position
 cudaError_t gm_prepare(int M);
 cudaError_t launch_chain_gm(ChainMode mode, const ChainArgs& a, float2* wv, int M, int* n_launches,

@@ -623,6 +623,8 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
   // Tables in FP64 on the host, rounded once to FP32.
   const int M = p.M;
   std::vector<float2> tw(M), hs(M);
+  std::vector<double> gain(M, 1.0);
+  if (!fused_window(M)) gm_factor_gain(M, gain.data());
   const double two_pi = 6.283185307179586476925287;
   for (int k = 0; k < M; ++k) {
     const double ang = -two_pi * (double)k / (double)M;
@@ -630,7 +632,8 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
     // fftfreq(M, pixel): k/(M*pixel) for k <= (M-1)/2, (k-M)/(M*pixel) otherwise (odd M too)
     const double f = (double)(k <= (M - 1) / 2 ? k : k - M) / ((double)M * p.pixel_A);
     const double ph = -M_PI * p.lambda_A * p.dz_A * f * f;
-    hs[k] = make_float2((float)(std::cos(ph) / M), (float)(std::sin(ph) / M));
+    const double norm = M * gain[k];
+    hs[k] = make_float2((float)(std::cos(ph) / norm), (float)(std::sin(ph) / norm));
   }
   // The full propagator h(ky) h(kx) / M^2 for the register-resident kernels.
   std::vector<float2> h2;
