@@ -33,6 +33,8 @@
 
 namespace ptycho {
 
+static_assert(kWaitExpired == PTYCHO_ERR_TIMEOUT, "the cluster's expired wait reports the library's code");
+
 namespace {
 
 // Elementwise over the pass-0 grouping (natural order), element (py, px).
@@ -96,7 +98,24 @@ __device__ __forceinline__ void store_patch(float2* p, float2 v) {
 
 template <int M, int MODE>
 __global__ void __launch_bounds__(Cfg<M>::T, Cfg<M>::MIN_BLOCKS) k_chain(const ChainArgs a) {
-  const int il = blockIdx.x;
+  using C = Cfg<M>;
+  const int il = blockIdx.x, t = threadIdx.x;
+#include "chain_body.inc"
+}
+
+// Few positions (Algorithm 1's per-location update, small batches, the last
+// partial wave of a chunk): one position per cluster of 8 blocks.  On one SM
+// its 16 warps take turns, 4 per scheduler, while most SMs idle; on 8 SMs each
+// warp has a scheduler to itself and what is left is the latency of a transform
+// (about 2.3 us, 4700 clocks).  Exchanges by cluster barriers and plain remote
+// stores took 184 us for one position of 16 slices, stores counted on the
+// receiver's mbarrier 168 us.
+template <int MODE>
+__global__ void __cluster_dims__(ClusterCfg128::CL, 1, 1) __launch_bounds__(ClusterCfg128::TB, 4)
+    k_chain_cluster(const ChainArgs a) {
+  using C = ClusterCfg128;
+  constexpr int M = C::M;
+  const int il = blockIdx.x / C::CL, t = (blockIdx.x % C::CL) * C::TB + threadIdx.x;
 #include "chain_body.inc"
 }
 
@@ -113,19 +132,22 @@ __global__ void __launch_bounds__(Cfg<M>::T, Cfg<M>::MIN_BLOCKS)
   if (threadIdx.x == 0) sa = m.a[p];
   __syncthreads();
   const ChainArgs& a = sa;
-  const int il = b - m.start[p];
+  using C = Cfg<M>;
+  const int il = b - m.start[p], t = threadIdx.x;
 #include "chain_body.inc"
 }
 
 int chain_threads(int M) { return M == 128 ? Cfg<128>::T : Cfg<64>::T; }
 
-size_t chain_smem_bytes(int M) {
-  // the exchange buffer, the pass-1 twiddle table, the loss partials of the
-  // warps and the tensor-memory address
-  const size_t tw1 = 16 * (size_t)(M == 128 ? tw1_stride<Cfg<128>>() : tw1_stride<Cfg<64>>());
-  return (size_t)M * M * sizeof(float2) + tw1 * sizeof(float2) + (size_t)(chain_threads(M) / 32) * sizeof(double) +
-         sizeof(double);
+// The exchange buffer, the pass-1 twiddle table, the loss partials of the
+// position's warps and the tensor-memory address.
+template <class C>
+static constexpr size_t chain_smem() {
+  return (C::kSmemWave + 16 * (size_t)tw1_stride<C>()) * sizeof(float2) + (C::T / 32 + 1) * sizeof(double) +
+         (C::CL > 1 ? 2 * sizeof(uint64_t) : 0);
 }
+
+size_t chain_smem_bytes(int M) { return M == 128 ? chain_smem<Cfg<128>>() : chain_smem<Cfg<64>>(); }
 
 template <int M>
 static cudaError_t prepare_m() {
@@ -165,8 +187,30 @@ static cudaError_t launch_m(ChainMode mode, const ChainArgs& a, cudaStream_t st)
   return cudaGetLastError();
 }
 
+static cudaError_t launch_cluster(ChainMode mode, const ChainArgs& a, cudaStream_t st) {
+  using C = ClusterCfg128;
+  const dim3 grid(a.n_pos * C::CL), block(C::TB);
+  const size_t smem = chain_smem<C>();
+  switch (mode) {
+    case MODE_FORWARD: k_chain_cluster<MODE_FORWARD><<<grid, block, smem, st>>>(a); break;
+    case MODE_LOSS: k_chain_cluster<MODE_LOSS><<<grid, block, smem, st>>>(a); break;
+    case MODE_GRAD_RC: k_chain_cluster<MODE_GRAD_RC><<<grid, block, smem, st>>>(a); break;
+    case MODE_RC_SEG: k_chain_cluster<MODE_RC_SEG><<<grid, block, smem, st>>>(a); break;
+    default: k_chain_cluster<MODE_GRAD><<<grid, block, smem, st>>>(a); break;
+  }
+  return cudaGetLastError();
+}
+
+// One launch of at most kClusterMax positions takes the cluster kernel (results
+// are the same bit for bit).  us of a gradient chain of 16 slices, one block
+// against one cluster per position: 1 position 311 -> 168, 10 311 -> 174, 19
+// 312 -> 205, 38 312 -> 255; with two blocks per SM and more the blocks of
+// different positions compete (76 positions 312 -> 520).
+constexpr int kClusterMax = 48;
+
 cudaError_t launch_chain(int M, ChainMode mode, const ChainArgs& a, cudaStream_t st) {
   if (a.n_pos <= 0) return cudaSuccess;
+  if (M == 128 && a.n_pos <= kClusterMax) return launch_cluster(mode, a, st);
   return M == 128 ? launch_m<128>(mode, a, st) : launch_m<64>(mode, a, st);
 }
 

@@ -167,12 +167,43 @@ __device__ __forceinline__ void dft_at(float2 (&v)[N]) {
 // that group sits at (py + a*SY(J), px + b*SX(J)).  swz() permutes columns
 // inside each 16-element block of a row (bank-conflict-free exchanges).
 // ---------------------------------------------------------------------------
+// Where a thread finds its per-pass factors (filled once per block by
+// fill_factors, every entry rounded once from FP64).  Read from shared and
+// global memory, each with its own index arithmetic, the twiddles and the
+// propagator were a third of the chain's shared-memory wavefronts and a fifth
+// of its instructions, and spilled registers.  A thread needs the same 2 V
+// pass-0 and spectrum factors for the whole chain, and tensor memory (unused
+// otherwise by this kernel) holds exactly 4 V = 128 words per thread and has a
+// data path of its own.  With the packed products below: one wave of 152
+// positions, M = 128, 16 slices 445 -> 380 us; 576 positions 2.20 -> 2.04 ms;
+// 960 positions, M = 64 1.06 -> 0.98 ms.  The adjoint now reads the exact
+// twiddles too (it multiplied two table entries per element before).
+//   tmem  this warp's 128 tensor-memory columns: words [0, 2V) hold the pass-0
+//         twiddles of the thread's V elements, words [2V, 4V) the propagator
+//         at its V spectrum elements (pass-2 grouping);
+//   tw1   shared table of the pass-1 twiddles, one row of G entries per
+//         (ey, ex) class (16 classes).
+struct Factors {
+  uint32_t tmem;
+  const float2* tw1;
+  // cluster only: the mbarriers of the two row buffers, the parity of their
+  // next completion, and the device error word
+  uint64_t* mbar = nullptr;
+  uint32_t phase = 0;
+  int* status = nullptr;
+};
+constexpr int kWaitExpired = -5;  // PTYCHO_ERR_TIMEOUT
+
 template <int M>
 struct Cfg;
 
 template <>
 struct Cfg<128> {
   static constexpr int M = 128, T = 512, V = 32, MIN_BLOCKS = 1;
+  static constexpr int CL = 1, TB = T, kSmemWave = M * M;  // blocks per position, threads per block
+  __device__ static __forceinline__ void sync() { __syncthreads(); }
+  __device__ static __forceinline__ void arrived(const Factors&, int) { __syncthreads(); }
+  __device__ static __forceinline__ void put_loss(double* red, int w, double v) { red[w] = v; }
   static constexpr int ry(int j) { return j == 0 ? 8 : 4; }
   static constexpr int rx(int j) { return j == 1 ? 8 : 4; }
   static constexpr int sy(int j) { return j == 0 ? 16 : (j == 1 ? 4 : 1); }
@@ -217,9 +248,60 @@ struct Cfg<128> {
   }
 };
 
+// The same wave over a cluster of 8 thread blocks of 64 threads (thread t of
+// the 512 is thread t % 64 of block t / 64), each on its own SM when few
+// positions run.  Block k owns the pass-1 and pass-2 groups of rows
+// 16 k .. 16 k + 15, so only the exchange between passes 0 and 1 crosses
+// blocks: forward, every element is stored into its pass-1 owner's row buffer;
+// inverse, into its pass-0 owner's.  The arithmetic of every element is that
+// of Cfg<128>, so results are bit-identical.
+struct ClusterCfg128 : Cfg<128> {
+  static constexpr int CL = 8, TB = T / CL, ROWS = M / CL;
+  static constexpr int kSmemWave = 2 * ROWS * M;  // float2: the two row buffers
+  __device__ static __forceinline__ void sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  __device__ static __forceinline__ void sync12(int) { __syncthreads(); }
+  __device__ static __forceinline__ void turn_wait(int) {}
+  __device__ static __forceinline__ void turn_pass(int) {}
+  // The exchanges need no cluster barrier: every store counts its bytes on the
+  // receiving buffer's mbarrier, and a block waits for its 16 KB.  A buffer may
+  // be written again once the exchange through the other one is complete: by
+  // then every block has sent, so has read what the first one held.
+  static constexpr uint32_t kBytes = ROWS * M * sizeof(float2);
+  static constexpr long long kWaitCycles = 2000000000LL;  // about 1 s
+  // address of p in block `rank` of the cluster
+  __device__ static __forceinline__ uint32_t peer(const void* p, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(tc::smem_u32(p)), "r"(rank));
+    return r;
+  }
+  __device__ static __forceinline__ void put(uint32_t addr, uint32_t mbar, float2 v) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr),
+                 "f"(v.x), "f"(v.y), "r"(mbar)
+                 : "memory");
+  }
+  // Buffer `which`'s exchange number `phase` has arrived.
+  __device__ static __forceinline__ void arrived(Factors& f, int which) {
+    uint64_t* mbar = f.mbar + which;
+    if (threadIdx.x == 0)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(mbar)), "r"(kBytes)
+                   : "memory");
+    if (!tc::mbar_wait_bounded(mbar, f.phase >> which & 1u, kWaitCycles)) *f.status = kWaitExpired;
+    f.phase ^= 1u << which;
+  }
+  __device__ static __forceinline__ void put_loss(double* red, int w, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(peer(red + w, 0)), "d"(v) : "memory");
+  }
+};
+
 template <>
 struct Cfg<64> {
   static constexpr int M = 64, T = 128, V = 32, MIN_BLOCKS = 4;
+  static constexpr int CL = 1, TB = T, kSmemWave = M * M;
+  __device__ static __forceinline__ void sync() { __syncthreads(); }
+  __device__ static __forceinline__ void arrived(const Factors&, int) { __syncthreads(); }
+  __device__ static __forceinline__ void put_loss(double* red, int w, double v) { red[w] = v; }
   static constexpr int ry(int) { return 4; }
   static constexpr int rx(int) { return 4; }
   static constexpr int sy(int j) { return j == 0 ? 16 : (j == 1 ? 4 : 1); }
@@ -271,8 +353,10 @@ __device__ __forceinline__ int opaque(int x) {
   return x;
 }
 
-template <class C, int J>
-__device__ __forceinline__ void xch_store(const float2 (&v)[C::V], float2* sm, int t) {
+// FAR: the exchange between passes 0 and 1 (the one that crosses the blocks of
+// a cluster; stored by pass 0 going forward and by pass 1 going back).
+template <class C, int J, bool FAR>
+__device__ __forceinline__ void xch_store(const float2 (&v)[C::V], float2* sm, const Factors& f, int t) {
   using P = PassShape<C, J>;
   t = opaque(t);
   static_for<0, P::Q>([&](auto qq) {
@@ -281,9 +365,23 @@ __device__ __forceinline__ void xch_store(const float2 (&v)[C::V], float2* sm, i
     C::template base<J>(t, q, py, px);
     static_for<0, P::RY>([&](auto aa) {
       constexpr int a = decltype(aa)::value;
+      const int y = py + a * P::SY;
+      [[maybe_unused]] uint32_t row = 0, mbar = 0;
+      if constexpr (C::CL > 1 && FAR) {  // into row buffer 0 by rows, or row buffer 1 by pass-0 owner
+        const int rank = J == 0 ? y / C::ROWS : y % 16 / 2;
+        row = C::peer(sm + (J == 0 ? y % C::ROWS : C::ROWS + y % 2 * 8 + y / 16) * C::M, rank);
+        mbar = C::peer(f.mbar + (J == 0 ? 0 : 1), rank);
+      }
       static_for<0, P::RX>([&](auto bb) {
         constexpr int b = decltype(bb)::value;
-        sm[(py + a * P::SY) * C::M + C::swz(px + b * P::SX)] = v[q * P::G + a * P::RX + b];
+        const int x = C::swz(px + b * P::SX);
+        const float2 e = v[q * P::G + a * P::RX + b];
+        if constexpr (C::CL == 1)
+          sm[y * C::M + x] = e;
+        else if constexpr (FAR)
+          C::put(row + 8 * x, mbar, e);
+        else
+          sm[(y % C::ROWS) * C::M + x] = e;
       });
     });
   });
@@ -299,34 +397,15 @@ __device__ __forceinline__ void xch_load(float2 (&v)[C::V], const float2* sm, in
     C::template base<J>(t, q, py, px);
     static_for<0, P::RY>([&](auto aa) {
       constexpr int a = decltype(aa)::value;
+      int y = py + a * P::SY;
+      if constexpr (C::CL > 1) y = J == 0 ? C::ROWS + y % 2 * 8 + y / 16 : y % C::ROWS;
       static_for<0, P::RX>([&](auto bb) {
         constexpr int b = decltype(bb)::value;
-        v[q * P::G + a * P::RX + b] = sm[(py + a * P::SY) * C::M + C::swz(px + b * P::SX)];
+        v[q * P::G + a * P::RX + b] = sm[y * C::M + C::swz(px + b * P::SX)];
       });
     });
   });
 }
-
-// Where a thread finds its per-pass factors (filled once per block by
-// fill_factors, every entry rounded once from FP64).  Read from shared and
-// global memory, each with its own index arithmetic, the twiddles and the
-// propagator were a third of the chain's shared-memory wavefronts and a fifth
-// of its instructions, and spilled registers.  A thread needs the same 2 V
-// pass-0 and spectrum factors for the whole chain, and tensor memory (unused
-// otherwise by this kernel) holds exactly 4 V = 128 words per thread and has a
-// data path of its own.  With the packed products below: one wave of 152
-// positions, M = 128, 16 slices 445 -> 380 us; 576 positions 2.20 -> 2.04 ms;
-// 960 positions, M = 64 1.06 -> 0.98 ms.  The adjoint now reads the exact
-// twiddles too (it multiplied two table entries per element before).
-//   tmem  this warp's 128 tensor-memory columns: words [0, 2V) hold the pass-0
-//         twiddles of the thread's V elements, words [2V, 4V) the propagator
-//         at its V spectrum elements (pass-2 grouping);
-//   tw1   shared table of the pass-1 twiddles, one row of G entries per
-//         (ey, ex) class (16 classes).
-struct Factors {
-  uint32_t tmem;
-  const float2* tw1;
-};
 
 template <class C>
 __host__ __device__ constexpr int tw1_stride() {  // float2; odd in 16-byte units: the classes fall on different banks
@@ -346,10 +425,65 @@ __device__ __forceinline__ void tmem_factors8(uint32_t taddr, float2 (&w)[8]) {
   for (int i = 0; i < 8; ++i) w[i] = make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
 }
 
+// All V complex values of the thread's tensor-memory words [word, word + 2V):
+// issued here, usable after tmem_factors_wait.
+__device__ __forceinline__ void tmem_factors_issue(uint32_t taddr, float2 (&w)[32]) {
+  static_for<0, 2>([&](auto hh) {
+    constexpr int h = decltype(hh)::value;
+    float2* p = w + 16 * h;
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=f"(p[0].x), "=f"(p[0].y), "=f"(p[1].x), "=f"(p[1].y), "=f"(p[2].x), "=f"(p[2].y), "=f"(p[3].x),
+          "=f"(p[3].y), "=f"(p[4].x), "=f"(p[4].y), "=f"(p[5].x), "=f"(p[5].y), "=f"(p[6].x), "=f"(p[6].y),
+          "=f"(p[7].x), "=f"(p[7].y), "=f"(p[8].x), "=f"(p[8].y), "=f"(p[9].x), "=f"(p[9].y), "=f"(p[10].x),
+          "=f"(p[10].y), "=f"(p[11].x), "=f"(p[11].y), "=f"(p[12].x), "=f"(p[12].y), "=f"(p[13].x), "=f"(p[13].y),
+          "=f"(p[14].x), "=f"(p[14].y), "=f"(p[15].x), "=f"(p[15].y)
+        : "r"(taddr + 32 * h));
+  });
+}
+__device__ __forceinline__ void tmem_factors_wait(float2 (&w)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(w[0].x), "+f"(w[0].y), "+f"(w[1].x), "+f"(w[1].y), "+f"(w[2].x), "+f"(w[2].y), "+f"(w[3].x),
+                 "+f"(w[3].y), "+f"(w[4].x), "+f"(w[4].y), "+f"(w[5].x), "+f"(w[5].y), "+f"(w[6].x), "+f"(w[6].y),
+                 "+f"(w[7].x), "+f"(w[7].y), "+f"(w[8].x), "+f"(w[8].y), "+f"(w[9].x), "+f"(w[9].y), "+f"(w[10].x),
+                 "+f"(w[10].y), "+f"(w[11].x), "+f"(w[11].y), "+f"(w[12].x), "+f"(w[12].y), "+f"(w[13].x),
+                 "+f"(w[13].y), "+f"(w[14].x), "+f"(w[14].y), "+f"(w[15].x), "+f"(w[15].y));
+  asm volatile("" : "+f"(w[16].x), "+f"(w[16].y), "+f"(w[17].x), "+f"(w[17].y), "+f"(w[18].x), "+f"(w[18].y),
+                    "+f"(w[19].x), "+f"(w[19].y), "+f"(w[20].x), "+f"(w[20].y), "+f"(w[21].x), "+f"(w[21].y),
+                    "+f"(w[22].x), "+f"(w[22].y), "+f"(w[23].x), "+f"(w[23].y), "+f"(w[24].x), "+f"(w[24].y),
+                    "+f"(w[25].x), "+f"(w[25].y), "+f"(w[26].x), "+f"(w[26].y), "+f"(w[27].x), "+f"(w[27].y),
+                    "+f"(w[28].x), "+f"(w[28].y), "+f"(w[29].x), "+f"(w[29].y), "+f"(w[30].x), "+f"(w[30].y),
+                    "+f"(w[31].x), "+f"(w[31].y));
+}
+template <bool CONJ, int FIRST_STEP>
+__device__ __forceinline__ void mul_factors(float2 (&v)[32], const float2 (&w)[32]) {
+  static_for<0, 32>([&](auto ee) {
+    constexpr int e = decltype(ee)::value;
+    if constexpr (e % FIRST_STEP != 0 || FIRST_STEP == 1) v[e] = pmul_opt<CONJ>(v[e], w[e]);
+  });
+}
+
 // One radix pass on the registers.  Forward: DFT over digit J of y (for every
 // x element), DFT over digit J of x (for every y element), then the twiddle
 // w_M^(ey*a' + ex*b') that couples digit J to the lower digits.  Inverse: the
 // conjugate twiddle, then the inverse DFTs (exact inverse up to the factor RY*RX).
+template <class C, int J, bool INV>
+__device__ __forceinline__ void pass_dft(float2 (&v)[C::V]) {
+  using P = PassShape<C, J>;
+  static_for<0, P::Q>([&](auto qq) {
+    constexpr int o = decltype(qq)::value * P::G;
+    static_for<0, P::RX>([&](auto bb) {
+      constexpr int b = decltype(bb)::value;
+      dft_at<P::RY, INV, o + b, P::RX>(v);
+    });
+    static_for<0, P::RY>([&](auto aa) {
+      constexpr int a = decltype(aa)::value;
+      dft_at<P::RX, INV, o + a * P::RX, 1>(v);
+    });
+  });
+}
+
 template <class C, int J, bool INV>
 __device__ __forceinline__ void pass_compute(float2 (&v)[C::V], const Factors& f, int t) {
   using P = PassShape<C, J>;
@@ -382,32 +516,32 @@ __device__ __forceinline__ void pass_compute(float2 (&v)[C::V], const Factors& f
     }
   };
   if constexpr (INV) twiddle();
-  static_for<0, P::Q>([&](auto qq) {
-    constexpr int o = decltype(qq)::value * P::G;
-    static_for<0, P::RX>([&](auto bb) {
-      constexpr int b = decltype(bb)::value;
-      dft_at<P::RY, INV, o + b, P::RX>(v);
-    });
-    static_for<0, P::RY>([&](auto aa) {
-      constexpr int a = decltype(aa)::value;
-      dft_at<P::RX, INV, o + a * P::RX, 1>(v);
-    });
-  });
+  pass_dft<C, J, INV>(v);
   if constexpr (!INV) twiddle();
 }
 
 // registers in pass-0 grouping (natural storage) -> unnormalised forward DFT,
-// registers in pass-2 grouping (digit-reversed storage)
+// registers in pass-2 grouping (digit-reversed storage).  The cluster's blocks
+// have registers to spare and only one warp per scheduler to hide latency, so
+// there the pass-0 twiddles are fetched whole while the wave is transformed.
 template <class C>
-__device__ __forceinline__ void fft_fwd(float2 (&v)[C::V], float2* sm, const Factors& f, int t) {
-  pass_compute<C, 0, false>(v, f, t);
-  xch_store<C, 0>(v, sm, t);
-  __syncthreads();
+__device__ __forceinline__ void fft_fwd(float2 (&v)[C::V], float2* sm, Factors& f, int t) {
+  if constexpr (C::CL > 1) {
+    float2 w[C::V];
+    tmem_factors_issue(f.tmem, w);
+    pass_dft<C, 0, false>(v);
+    tmem_factors_wait(w);
+    mul_factors<false, PassShape<C, 0>::G>(v, w);
+  } else {
+    pass_compute<C, 0, false>(v, f, t);
+  }
+  xch_store<C, 0, true>(v, sm, f, t);
+  C::arrived(f, 0);
   C::turn_wait(t);
   xch_load<C, 1>(v, sm, t);
   C::turn_pass(t);
   pass_compute<C, 1, false>(v, f, t);
-  xch_store<C, 1>(v, sm, t);
+  xch_store<C, 1, false>(v, sm, f, t);
   C::sync12(t);
   xch_load<C, 2>(v, sm, t);
   pass_compute<C, 2, false>(v, f, t);
@@ -416,24 +550,41 @@ __device__ __forceinline__ void fft_fwd(float2 (&v)[C::V], float2* sm, const Fac
 // exact reverse of fft_fwd: unnormalised inverse DFT (times M*M relative to
 // the true inverse), registers back in pass-0 grouping
 template <class C>
-__device__ __forceinline__ void fft_inv(float2 (&v)[C::V], float2* sm, const Factors& f, int t) {
+__device__ __forceinline__ void fft_inv(float2 (&v)[C::V], float2* sm, Factors& f, int t) {
   pass_compute<C, 2, true>(v, f, t);
-  xch_store<C, 2>(v, sm, t);
+  xch_store<C, 2, false>(v, sm, f, t);
   C::sync12(t);
   xch_load<C, 1>(v, sm, t);
   pass_compute<C, 1, true>(v, f, t);
-  xch_store<C, 1>(v, sm, t);
-  __syncthreads();
-  C::turn_wait(t);
-  xch_load<C, 0>(v, sm, t);
-  C::turn_pass(t);
-  pass_compute<C, 0, true>(v, f, t);
+  xch_store<C, 1, true>(v, sm, f, t);
+  if constexpr (C::CL > 1) {
+    float2 w[C::V];
+    tmem_factors_issue(f.tmem, w);
+    C::arrived(f, 1);
+    xch_load<C, 0>(v, sm, t);
+    tmem_factors_wait(w);
+    mul_factors<true, PassShape<C, 0>::G>(v, w);
+    pass_dft<C, 0, true>(v);
+  } else {
+    C::arrived(f, 1);
+    C::turn_wait(t);
+    xch_load<C, 0>(v, sm, t);
+    C::turn_pass(t);
+    pass_compute<C, 0, true>(v, f, t);
+  }
 }
 
 // Multiply the spectrum (pass-2 grouping) by the propagator h(ky, kx) / M^2 or
 // its conjugate.
 template <class C, bool CONJ>
 __device__ __forceinline__ void mul_prop(float2 (&v)[C::V], const Factors& f) {
+  if constexpr (C::CL > 1) {
+    float2 w[C::V];
+    tmem_factors_issue(f.tmem + 2 * C::V, w);
+    tmem_factors_wait(w);
+    mul_factors<CONJ, 1>(v, w);
+    return;
+  }
   static_for<0, C::V / 8>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
     float2 w[8];
@@ -452,10 +603,10 @@ __device__ __forceinline__ void mul_prop(float2 (&v)[C::V], const Factors& f) {
 template <class C>
 __device__ __forceinline__ void fill_factors(uint32_t taddr, float2* tw1, const float2* __restrict__ tw,
                                              const float2* __restrict__ h2, bool with_h, int t) {
-  {
+  {  // (each block of a cluster keeps the whole table)
     using P = PassShape<C, 1>;
     constexpr int EY = C::M / (P::RY * P::SY), EX = C::M / (P::RX * P::SX);
-    for (int k = t; k < P::SY * P::SX * P::G; k += C::T) {
+    for (int k = t % C::TB; k < P::SY * P::SX * P::G; k += C::TB) {
       const int cls = k / P::G, e = k % P::G;
       const int ex = EY * (cls / P::SX) * (e / P::RX) + EX * (cls % P::SX) * (e % P::RX);
       tw1[cls * tw1_stride<C>() + e] = __ldg(tw + (ex & (C::M - 1)));
