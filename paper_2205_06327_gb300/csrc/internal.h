@@ -103,12 +103,24 @@ struct AccumArgs {
                             // ws_gphi slot s (every wave kept)
 };
 cudaError_t launch_accum_obj_grad(const AccumArgs& a, cudaStream_t st);
-cudaError_t launch_probe_grad(const float2* ws_gp, int n_pos, int M, float2* part, int n_split,
-                              float2* grad_probe, int accumulate, cudaStream_t st);
+// Probe gradient (sum of ws_gp over the positions) and loss of one chunk.
+cudaError_t launch_probe_loss(const float2* ws_gp, int n_pos, int M, float2* part, int n_split, float2* grad_probe,
+                              const double* loss_part, int n_loss, double* loss, int accumulate, int* n_launches,
+                              cudaStream_t st);
 cudaError_t launch_loss_accum(const double* loss_part, int n, double* acc, int accumulate,
                               cudaStream_t st);
-cudaError_t launch_axpy(float2* y, const float2* x, const float2* base, double alpha, size_t n,
-                        cudaStream_t st);  // y = base + alpha * x
+struct UpdateArgs {
+  float2* obj;            // += a_obj g_obj
+  const float2* g_obj;
+  size_t n_obj;
+  float2* probe;          // += a_probe g_probe
+  const float2* g_probe;
+  size_t n_probe;
+  float a_obj, a_probe;
+  float2* acc;            // null, or += g_obj
+  int flush;              // with acc: obj += a_obj acc, acc = 0
+};
+cudaError_t launch_update(const UpdateArgs& u, cudaStream_t st);
 cudaError_t launch_norm2(const float2* x, size_t n, double* part, int n_part, double* out,
                          int slot, cudaStream_t st);
 cudaError_t launch_potential_to_transmission(const float* V, float2* O, double sigma, size_t n, cudaStream_t st);

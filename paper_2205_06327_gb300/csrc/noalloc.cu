@@ -216,12 +216,11 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
       g.accumulate = ci > 0;
       if ((e = launch_accum_obj_grad(g, st)) != cudaSuccess) return noalloc_fail(PTYCHO_ERR_CUDA, cudaGetErrorString(e));
     }
-    if (grad_probe &&
-        (e = launch_probe_grad(ws_gp, n, M, gp_part, kSplit, reinterpret_cast<float2*>(grad_probe), ci > 0, st)) !=
-            cudaSuccess)
-      return noalloc_fail(PTYCHO_ERR_CUDA, cudaGetErrorString(e));
-    if ((e = launch_loss_accum(loss_part, n, d_loss, ci > 0, st)) != cudaSuccess)
-      return noalloc_fail(PTYCHO_ERR_CUDA, cudaGetErrorString(e));
+    int launches = 0;
+    e = grad_probe ? launch_probe_loss(ws_gp, n, M, gp_part, kSplit, reinterpret_cast<float2*>(grad_probe), loss_part,
+                                       n, d_loss, ci > 0, &launches, st)
+                   : launch_loss_accum(loss_part, n, d_loss, ci > 0, st);
+    if (e != cudaSuccess) return noalloc_fail(PTYCHO_ERR_CUDA, cudaGetErrorString(e));
   }
 
   // The call is synchronous: it waits for the stream to report the status.

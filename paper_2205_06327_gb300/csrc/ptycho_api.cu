@@ -432,6 +432,33 @@ int accum_part(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, floa
   return PTYCHO_OK;
 }
 
+// Probe gradient (unless null) and loss of the chunk's n positions.
+int finish_chunk(ptycho_plan pl, int n, float2* grad_probe, int slot, int accumulate, cudaStream_t st) {
+  const int n_loss = n * pl->loss_parts;
+  if (!grad_probe) {
+    TIMED(K_OTHER, 1, launch_loss_accum(pl->loss_part, n_loss, pl->d_scal + slot, accumulate, st));
+    return PTYCHO_OK;
+  }
+  int launches = 0;
+  TIMED(K_PROBE, 0,
+        launch_probe_loss(pl->ws_gp, n, pl->p.M, pl->gp_part, kProbeSplit, grad_probe, pl->loss_part, n_loss,
+                          pl->d_scal + slot, accumulate, &launches, st));
+  pl->tm.launches += launches;
+  return PTYCHO_OK;
+}
+
+// O += a_o dF/dO and P += a_p dF/dP from the plan's step buffers; with acc,
+// the delayed accumulation (see ptycho_step_accumulate).
+int update_step(ptycho_plan pl, ptycho_c64* obj, ptycho_c64* probe, double a_o, double a_p, ptycho_c64* acc, int flush,
+                cudaStream_t st) {
+  const ptycho_params& p = pl->p;
+  const UpdateArgs u{reinterpret_cast<float2*>(obj), pl->g_obj, (size_t)p.S * p.H * p.W,
+                     reinterpret_cast<float2*>(probe), pl->g_probe, (size_t)p.M * p.M, (float)a_o, (float)a_p,
+                     reinterpret_cast<float2*>(acc), flush};
+  TIMED(K_OTHER, 1, launch_update(u, st));
+  return PTYCHO_OK;
+}
+
 // F (and optionally gradients) at (probe + probe_step*probe_dir, obj + obj_step*obj_dir);
 // the loss lands in pl->d_scal[slot].  With rest_ready, only the intensities
 // of the first n_first positions are ready when the call starts: the chain of
@@ -570,9 +597,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
     } else if (grad_obj) {
       if ((rc = accum_for(c0, 0, n, ci > 0, st)) != PTYCHO_OK) return rc;
     }
-    if (grad_probe)
-      TIMED(K_PROBE, 2, launch_probe_grad(pl->ws_gp, n, p.M, pl->gp_part, kProbeSplit, grad_probe, ci > 0, st));
-    TIMED(K_OTHER, 1, launch_loss_accum(pl->loss_part, n * pl->loss_parts, pl->d_scal + slot, ci > 0, st));
+    if ((rc = finish_chunk(pl, n, grad_probe, slot, ci > 0, st))) return rc;
   }
   return PTYCHO_OK;
 }
@@ -852,7 +877,7 @@ int loss_grad_impl(ptycho_plan plan, const int32_t* pos_yx, const ptycho_c64* pr
 
 int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho_c64* obj, const float* meas_I,
               double alpha_obj, double alpha_probe, int32_t line_search, double* loss_out, double* t_out,
-              cudaStream_t st) {
+              cudaStream_t st, ptycho_c64* acc = nullptr, int flush = 0) {
   if (!plan) return fail(PTYCHO_ERR_ARG, "plan is NULL");
   if (!std::isfinite(alpha_obj) || !std::isfinite(alpha_probe))
     return fail(PTYCHO_ERR_ARG, "step sizes must be finite");
@@ -868,8 +893,6 @@ int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho
   rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, plan->g_obj, plan->g_probe, 0, nullptr, 0.f, nullptr, 0.f, st);
   if (rc) return rc;
   if ((rc = deliver_loss(plan, 0, loss_out, st))) return rc;
-  float2* O = reinterpret_cast<float2*>(obj);
-  float2* P = reinterpret_cast<float2*>(probe);
   ptycho_plan pl = plan;
   double t = 1.0;
   if (line_search) {
@@ -894,10 +917,7 @@ int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho
     }
     if (!accepted) t = 0.0;
   }
-  if (t > 0.0) {
-    TIMED(K_OTHER, 1, launch_axpy(O, plan->g_obj, O, -t * alpha_obj, nO, st));
-    TIMED(K_OTHER, 1, launch_axpy(P, plan->g_probe, P, -t * alpha_probe, nP, st));
-  }
+  if (t > 0.0 && (rc = update_step(plan, obj, probe, -t * alpha_obj, -t * alpha_probe, acc, flush, st))) return rc;
   if (t_out) *t_out = t;
   return PTYCHO_OK;
 }
@@ -1012,9 +1032,8 @@ int run_multi_fused(const ptycho_problem* probs, const std::vector<int>& idx, bo
           if ((rc = accum_part(pl, q.pos_yx, q.probe, it->gO, c0, 0, n - tail, r > 0, st))) return rc;
           if (tail && (rc = accum_part(pl, q.pos_yx, q.probe, it->gO, c0, n - tail, tail, 1, st))) return rc;
         }
-        if (it->gP)
-          TIMED(K_PROBE, 2, launch_probe_grad(pl->ws_gp, n, pl->p.M, pl->gp_part, kProbeSplit, it->gP, r > 0, st));
-        TIMED(K_OTHER, 1, launch_loss_accum(pl->loss_part, n, pl->d_scal, r > 0, st));
+        int rc;
+        if ((rc = finish_chunk(pl, n, it->gP, 0, r > 0, st))) return rc;
       }
     }
   }
@@ -1023,13 +1042,7 @@ int run_multi_fused(const ptycho_problem* probs, const std::vector<int>& idx, bo
     const ptycho_problem& q = probs[it.i];
     int rc;
     if ((rc = deliver_loss(pl, 0, q.loss_out, st))) return rc;
-    if (step) {
-      const ptycho_params& p = pl->p;
-      TIMED(K_OTHER, 1, launch_axpy(reinterpret_cast<float2*>(q.obj), pl->g_obj, reinterpret_cast<float2*>(q.obj),
-                                    -a_o, (size_t)p.S * p.H * p.W, st));
-      TIMED(K_OTHER, 1, launch_axpy(reinterpret_cast<float2*>(q.probe), pl->g_probe,
-                                    reinterpret_cast<float2*>(q.probe), -a_p, (size_t)p.M * p.M, st));
-    }
+    if (step && (rc = update_step(pl, q.obj, q.probe, -a_o, -a_p, nullptr, 0, st))) return rc;
   }
   return PTYCHO_OK;
 }
@@ -1161,20 +1174,8 @@ int ptycho_step_accumulate(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* 
   int rc;
   if ((rc = check_array(acc, "acc", true))) return rc;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if ((rc = step_impl(plan, pos_yx, probe, obj, meas_I, alpha_obj, alpha_probe, 0, loss_out, nullptr, st)))
-    return rc;
-  // step_impl left this call's object gradient in the plan's step buffer
-  const ptycho_params& p = plan->p;
-  const size_t nO = (size_t)p.S * p.H * p.W;
-  float2* A = reinterpret_cast<float2*>(acc);
-  float2* O = reinterpret_cast<float2*>(obj);
-  ptycho_plan pl = plan;
-  TIMED_ON(st, K_OTHER, 1, launch_axpy(A, plan->g_obj, A, 1.0, nO, st));  // AccBuf += dF/dO
-  if (flush) {
-    TIMED_ON(st, K_OTHER, 1, launch_axpy(O, A, O, -alpha_obj, nO, st));  // second update
-    CUDA_TRY(cudaMemsetAsync(A, 0, nO * sizeof(float2), st));
-  }
-  return PTYCHO_OK;
+  return step_impl(plan, pos_yx, probe, obj, meas_I, alpha_obj, alpha_probe, 0, loss_out, nullptr, st, acc,
+                   flush ? 1 : 0);
 }
 
 int ptycho_multi_loss_grad(const ptycho_problem* problems, int32_t n, void* stream) {

@@ -233,21 +233,8 @@ __global__ void k_probe_grad_part(const float2* __restrict__ ws_gp, int n_pos, i
   part[(size_t)sp * MM + pix] = acc;
 }
 
-__global__ void k_probe_grad_final(const float2* __restrict__ part, int MM, int n_split,
-                                   float2* __restrict__ gp, int accumulate) {
-  const int pix = blockIdx.x * blockDim.x + threadIdx.x;
-  if (pix >= MM) return;
-  float2 acc = accumulate ? gp[pix] : make_float2(0.f, 0.f);
-  for (int sp = 0; sp < n_split; ++sp) {
-    const float2 g = part[(size_t)sp * MM + pix];
-    acc.x += g.x;
-    acc.y += g.y;
-  }
-  gp[pix] = acc;
-}
-
-// Fixed-order FP64 sum of n values into acc[0] (one block).
-__global__ void k_loss_accum(const double* __restrict__ part, int n, double* acc, int accumulate) {
+// Fixed-order FP64 sum of n values into acc[0] (one block of 256 threads).
+__device__ __forceinline__ void loss_sum(const double* __restrict__ part, int n, double* acc, int accumulate) {
   __shared__ double sh[256];
   const int t = threadIdx.x;
   double s = 0.0;
@@ -261,10 +248,70 @@ __global__ void k_loss_accum(const double* __restrict__ part, int n, double* acc
   if (t == 0) acc[0] = (accumulate ? acc[0] : 0.0) + sh[0];
 }
 
-__global__ void k_axpy(float2* y, const float2* __restrict__ x, const float2* base, float alpha, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float2 b = base[i], d = x[i];
-    y[i] = make_float2(fmaf(alpha, d.x, b.x), fmaf(alpha, d.y, b.y));
+__global__ void k_loss_accum(const double* __restrict__ part, int n, double* acc, int accumulate) {
+  loss_sum(part, n, acc, accumulate);
+}
+
+// The end of an evaluation in one launch: the probe gradient's splits and, in
+// one more block, the loss.  PER > 0 (splits of at most PER positions, few
+// positions): sums the positions of each split here, in the order of
+// k_probe_grad_part, so that its launch falls away too.
+template <int PER>
+__global__ void __launch_bounds__(256) k_probe_loss(const float2* __restrict__ src, int n, int MM,
+                                                    float2* __restrict__ gp, const double* __restrict__ loss_part,
+                                                    int n_loss, double* loss, int accumulate) {
+  if (blockIdx.x == gridDim.x - 1) {
+    loss_sum(loss_part, n_loss, loss, accumulate);
+    return;
+  }
+  const int pix = blockIdx.x * 256 + threadIdx.x;
+  if (pix >= MM) return;
+  constexpr int U = 8, P = PER > 0 ? PER : 1;
+  float2 acc = accumulate ? gp[pix] : make_float2(0.f, 0.f);
+  for (int i0 = 0; i0 < n; i0 += U) {
+    float2 g[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      g[u] = i0 + u < n ? __ldcs(src + (size_t)(i0 + u) * MM + pix) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < U; u += P) {
+      float2 part = g[u];
+#pragma unroll
+      for (int k = 1; k < P; ++k) {
+        part.x += g[u + k].x;
+        part.y += g[u + k].y;
+      }
+      acc.x += part.x;
+      acc.y += part.y;
+    }
+  }
+  gp[pix] = acc;
+}
+
+// The update of a step in one launch: O += a_o dF/dO, P += a_p dF/dP, and for
+// the delayed accumulation (ACC) acc += dF/dO and, with `flush`, the second
+// update O += a_o acc, acc = 0.
+template <bool ACC>
+__global__ void __launch_bounds__(256) k_update(const UpdateArgs u) {
+  const size_t stride = (size_t)gridDim.x * 256;
+  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < u.n_obj; i += stride) {
+    const float2 d = u.g_obj[i];
+    float2 o = u.obj[i];
+    o = make_float2(fmaf(u.a_obj, d.x, o.x), fmaf(u.a_obj, d.y, o.y));
+    if constexpr (ACC) {
+      float2 c = u.acc[i];
+      c = make_float2(c.x + d.x, c.y + d.y);
+      if (u.flush) {
+        o = make_float2(fmaf(u.a_obj, c.x, o.x), fmaf(u.a_obj, c.y, o.y));
+        c = make_float2(0.f, 0.f);
+      }
+      u.acc[i] = c;
+    }
+    u.obj[i] = o;
+  }
+  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < u.n_probe; i += stride) {
+    const float2 d = u.g_probe[i], p = u.probe[i];
+    u.probe[i] = make_float2(fmaf(u.a_probe, d.x, p.x), fmaf(u.a_probe, d.y, p.y));
   }
 }
 
@@ -375,12 +422,20 @@ cudaError_t launch_accum_obj_grad(const AccumArgs& args, cudaStream_t st) {
   return vec == 2 ? accum_steps<2>(steps, a, grid, st) : accum_steps<1>(steps, a, grid, st);
 }
 
-cudaError_t launch_probe_grad(const float2* ws_gp, int n_pos, int M, float2* part, int n_split,
-                              float2* grad_probe, int accumulate, cudaStream_t st) {
-  const int MM = M * M;
-  const dim3 g1((MM + 255) / 256, n_split);
-  k_probe_grad_part<<<g1, 256, 0, st>>>(ws_gp, n_pos, MM, n_split, part);
-  k_probe_grad_final<<<(MM + 255) / 256, 256, 0, st>>>(part, MM, n_split, grad_probe, accumulate);
+cudaError_t launch_probe_loss(const float2* ws_gp, int n_pos, int M, float2* part, int n_split, float2* grad_probe,
+                              const double* loss_part, int n_loss, double* loss, int accumulate, int* n_launches,
+                              cudaStream_t st) {
+  const int MM = M * M, blocks = (MM + 255) / 256;
+  *n_launches = 1;
+  if (n_pos <= n_split) {
+    k_probe_loss<1><<<blocks + 1, 256, 0, st>>>(ws_gp, n_pos, MM, grad_probe, loss_part, n_loss, loss, accumulate);
+  } else if (n_pos <= 2 * n_split) {
+    k_probe_loss<2><<<blocks + 1, 256, 0, st>>>(ws_gp, n_pos, MM, grad_probe, loss_part, n_loss, loss, accumulate);
+  } else {
+    *n_launches = 2;
+    k_probe_grad_part<<<dim3(blocks, n_split), 256, 0, st>>>(ws_gp, n_pos, MM, n_split, part);
+    k_probe_loss<0><<<blocks + 1, 256, 0, st>>>(part, n_split, MM, grad_probe, loss_part, n_loss, loss, accumulate);
+  }
   return cudaGetLastError();
 }
 
@@ -389,10 +444,15 @@ cudaError_t launch_loss_accum(const double* loss_part, int n, double* acc, int a
   return cudaGetLastError();
 }
 
-cudaError_t launch_axpy(float2* y, const float2* x, const float2* base, double alpha, size_t n, cudaStream_t st) {
+cudaError_t launch_update(const UpdateArgs& u, cudaStream_t st) {
+  const size_t n = u.n_obj > u.n_probe ? u.n_obj : u.n_probe;
   if (n == 0) return cudaSuccess;
   const size_t blocks = (n + 255) / 256;
-  k_axpy<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, st>>>(y, x, base, (float)alpha, n);
+  const unsigned grid = (unsigned)(blocks < 4096 ? blocks : 4096);
+  if (u.acc)
+    k_update<true><<<grid, 256, 0, st>>>(u);
+  else
+    k_update<false><<<grid, 256, 0, st>>>(u);
   return cudaGetLastError();
 }
 
