@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(kGmThreads, 4)
     }
     for (int k = t; k < M; k += kGmThreads) H[k] = a.hs[k];
   }
+  dependency_wait();
   const int il = blockIdx.x / parts, part = blockIdx.x % parts;
   const GmBlock b{a, g, M, part * L, il, a.pos[a.pos_begin + il], g.cols != 0};
   if (!window_ok(b.r, M, a.H, a.W)) {
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(kGmThreads, 4)
     if (g.op2 == GM_PROP) propagate();
     if (g.op2 == GM_FFT) transform(std::false_type{});
   }
+  launch_dependents();
   float2* dst = g.dst + (size_t)il * M * M;
   each([&](int li, int i) { dst[b.at(li, i)] = x[li * LS + gm_pad(i)]; });
 }
@@ -358,13 +360,9 @@ struct GmLauncher {
     const int L = gm_lines(M);
     const unsigned grid = (unsigned)((size_t)a.n_pos * (M / L));
     const size_t smem = gm_rt_smem(M);
-    if (kind == GM_FWD)
-      k_gm_pass_rt<GM_FWD><<<grid, kGmThreads, smem, st>>>(a, g, M, L, plan);
-    else if (kind == GM_ADJ)
-      k_gm_pass_rt<GM_ADJ><<<grid, kGmThreads, smem, st>>>(a, g, M, L, plan);
-    else
-      k_gm_pass_rt<GM_RES><<<grid, kGmThreads, smem, st>>>(a, g, M, L, plan);
-    return cudaGetLastError();
+    void (*k)(ChainArgs, GmPass, int, int, GmPlan) =
+        kind == GM_FWD ? k_gm_pass_rt<GM_FWD> : kind == GM_ADJ ? k_gm_pass_rt<GM_ADJ> : k_gm_pass_rt<GM_RES>;
+    return launch_after(k, grid, kGmThreads, smem, st, a, g, M, L, plan);
   }
 };
 

@@ -178,13 +178,12 @@ static cudaError_t launch_m(ChainMode mode, const ChainArgs& a, cudaStream_t st)
   const dim3 grid(a.n_pos), block(Cfg<M>::T);
   const size_t smem = chain_smem_bytes(M);
   switch (mode) {
-    case MODE_FORWARD: k_chain<M, MODE_FORWARD><<<grid, block, smem, st>>>(a); break;
-    case MODE_LOSS: k_chain<M, MODE_LOSS><<<grid, block, smem, st>>>(a); break;
-    case MODE_GRAD_RC: k_chain<M, MODE_GRAD_RC><<<grid, block, smem, st>>>(a); break;
-    case MODE_RC_SEG: k_chain<M, MODE_RC_SEG><<<grid, block, smem, st>>>(a); break;
-    default: k_chain<M, MODE_GRAD><<<grid, block, smem, st>>>(a); break;
+    case MODE_FORWARD: return launch_after(k_chain<M, MODE_FORWARD>, grid, block, smem, st, a);
+    case MODE_LOSS: return launch_after(k_chain<M, MODE_LOSS>, grid, block, smem, st, a);
+    case MODE_GRAD_RC: return launch_after(k_chain<M, MODE_GRAD_RC>, grid, block, smem, st, a);
+    case MODE_RC_SEG: return launch_after(k_chain<M, MODE_RC_SEG>, grid, block, smem, st, a);
+    default: return launch_after(k_chain<M, MODE_GRAD>, grid, block, smem, st, a);
   }
-  return cudaGetLastError();
 }
 
 static cudaError_t launch_cluster(ChainMode mode, const ChainArgs& a, cudaStream_t st) {
@@ -192,13 +191,12 @@ static cudaError_t launch_cluster(ChainMode mode, const ChainArgs& a, cudaStream
   const dim3 grid(a.n_pos * C::CL), block(C::TB);
   const size_t smem = chain_smem<C>();
   switch (mode) {
-    case MODE_FORWARD: k_chain_cluster<MODE_FORWARD><<<grid, block, smem, st>>>(a); break;
-    case MODE_LOSS: k_chain_cluster<MODE_LOSS><<<grid, block, smem, st>>>(a); break;
-    case MODE_GRAD_RC: k_chain_cluster<MODE_GRAD_RC><<<grid, block, smem, st>>>(a); break;
-    case MODE_RC_SEG: k_chain_cluster<MODE_RC_SEG><<<grid, block, smem, st>>>(a); break;
-    default: k_chain_cluster<MODE_GRAD><<<grid, block, smem, st>>>(a); break;
+    case MODE_FORWARD: return launch_after(k_chain_cluster<MODE_FORWARD>, grid, block, smem, st, a);
+    case MODE_LOSS: return launch_after(k_chain_cluster<MODE_LOSS>, grid, block, smem, st, a);
+    case MODE_GRAD_RC: return launch_after(k_chain_cluster<MODE_GRAD_RC>, grid, block, smem, st, a);
+    case MODE_RC_SEG: return launch_after(k_chain_cluster<MODE_RC_SEG>, grid, block, smem, st, a);
+    default: return launch_after(k_chain_cluster<MODE_GRAD>, grid, block, smem, st, a);
   }
-  return cudaGetLastError();
 }
 
 // One launch of at most kClusterMax positions takes the cluster kernel (results
@@ -219,11 +217,8 @@ cudaError_t launch_chain_multi(int M, const MultiChainArgs& m, cudaStream_t st) 
   if (m.n == 0 || m.start[m.n] <= 0) return cudaSuccess;
   const dim3 grid(m.start[m.n]), block(chain_threads(M));
   const size_t smem = chain_smem_bytes(M);
-  if (M == 128)
-    k_chain_multi<128><<<grid, block, smem, st>>>(m);
-  else
-    k_chain_multi<64><<<grid, block, smem, st>>>(m);
-  return cudaGetLastError();
+  return M == 128 ? launch_after(k_chain_multi<128>, grid, block, smem, st, m)
+                  : launch_after(k_chain_multi<64>, grid, block, smem, st, m);
 }
 
 }  // namespace ptycho

@@ -7,6 +7,30 @@
 
 namespace ptycho {
 
+// Programmatic dependent launch: a kernel launched with launch_after may start
+// once every block of the kernel before it in the stream has called
+// launch_dependents (or ended), and fill its tables while that one still runs.
+// dependency_wait returns when the kernel before it is complete and its writes
+// are visible: every such kernel calls it before it touches anything but
+// constant tables, so completion carries over from kernel to kernel.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // MODE_GRAD stores every slice's entering wave and exit-wave gradient.
 // Recompute mode (checkpoint every ckpt_L slices, K segments) is K launches:
 // MODE_GRAD_RC runs the forward model keeping the checkpoints and the last

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumAr
   __shared__ int wcount[kAccWarps];
   extern __shared__ float2 acc[];  // [8][2 acc_half(tile_w)]: a row's even columns, then its odd ones
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  dependency_wait();
   const int z = blockIdx.x % a.n_slices, b = blockIdx.x / a.n_slices;  // slice s_begin + z
   const int s = a.s_begin + z;
   const int M = a.M;
@@ -229,6 +230,8 @@ __global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumAr
 // part[sp][pix] = sum over positions of split sp (ascending) of ws_gp[i][pix]
 __global__ void k_probe_grad_part(const float2* __restrict__ ws_gp, int n_pos, int MM, int n_split,
                                   float2* __restrict__ part) {
+  launch_dependents();
+  dependency_wait();
   const int pix = blockIdx.x * blockDim.x + threadIdx.x;
   const int sp = blockIdx.y;
   if (pix >= MM) return;
@@ -259,6 +262,8 @@ __device__ __forceinline__ void loss_sum(const double* __restrict__ part, int n,
 }
 
 __global__ void k_loss_accum(const double* __restrict__ part, int n, double* acc, int accumulate) {
+  launch_dependents();
+  dependency_wait();
   loss_sum(part, n, acc, accumulate);
 }
 
@@ -270,6 +275,8 @@ template <int PER>
 __global__ void __launch_bounds__(256) k_probe_loss(const float2* __restrict__ src, int n, int MM,
                                                     float2* __restrict__ gp, const double* __restrict__ loss_part,
                                                     int n_loss, double* loss, int accumulate) {
+  launch_dependents();
+  dependency_wait();
   if (blockIdx.x == gridDim.x - 1) {
     loss_sum(loss_part, n_loss, loss, accumulate);
     return;
@@ -303,6 +310,8 @@ __global__ void __launch_bounds__(256) k_probe_loss(const float2* __restrict__ s
 // update O += a_o acc, acc = 0.
 template <bool ACC>
 __global__ void __launch_bounds__(256) k_update(const UpdateArgs u) {
+  launch_dependents();
+  dependency_wait();
   const size_t stride = (size_t)gridDim.x * 256;
   for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < u.n_obj; i += stride) {
     const float2 d = u.g_obj[i];
@@ -376,14 +385,13 @@ namespace {
 template <int K, int VEC>
 cudaError_t accum_launch(const AccumArgs& a, dim3 grid, cudaStream_t st) {
   const size_t smem = (size_t)kAccWarps * 2 * acc_half(a.tile_w) * sizeof(float2);
-  const auto k = a.patch_mode ? k_accum_obj_grad<K, VEC, true> : k_accum_obj_grad<K, VEC, false>;
+  void (*const k)(AccumArgs) = a.patch_mode ? k_accum_obj_grad<K, VEC, true> : k_accum_obj_grad<K, VEC, false>;
   if (smem > 2 * acc_half(kAccDefaultCols) * kAccWarps * sizeof(float2)) {  // beyond the 48 KB every kernel may use
     const cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * acc_half(kAccMaxCols) * kAccWarps * (int)sizeof(float2));
     if (e != cudaSuccess) return e;
   }
-  k<<<grid, kAccThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_after(k, grid, kAccThreads, smem, st, a);
 }
 
 template <int VEC>
@@ -437,21 +445,23 @@ cudaError_t launch_probe_loss(const float2* ws_gp, int n_pos, int M, float2* par
                               cudaStream_t st) {
   const int MM = M * M, blocks = (MM + 255) / 256;
   *n_launches = 1;
-  if (n_pos <= n_split) {
-    k_probe_loss<1><<<blocks + 1, 256, 0, st>>>(ws_gp, n_pos, MM, grad_probe, loss_part, n_loss, loss, accumulate);
-  } else if (n_pos <= 2 * n_split) {
-    k_probe_loss<2><<<blocks + 1, 256, 0, st>>>(ws_gp, n_pos, MM, grad_probe, loss_part, n_loss, loss, accumulate);
-  } else {
+  const float2* src = ws_gp;
+  int n = n_pos;
+  void (*k)(const float2*, int, int, float2*, const double*, int, double*, int) =
+      n_pos <= n_split ? k_probe_loss<1> : n_pos <= 2 * n_split ? k_probe_loss<2> : k_probe_loss<0>;
+  if (n_pos > 2 * n_split) {
     *n_launches = 2;
-    k_probe_grad_part<<<dim3(blocks, n_split), 256, 0, st>>>(ws_gp, n_pos, MM, n_split, part);
-    k_probe_loss<0><<<blocks + 1, 256, 0, st>>>(part, n_split, MM, grad_probe, loss_part, n_loss, loss, accumulate);
+    const cudaError_t e =
+        launch_after(k_probe_grad_part, dim3(blocks, n_split), 256, 0, st, ws_gp, n_pos, MM, n_split, part);
+    if (e != cudaSuccess) return e;
+    src = part;
+    n = n_split;
   }
-  return cudaGetLastError();
+  return launch_after(k, blocks + 1, 256, 0, st, src, n, MM, grad_probe, loss_part, n_loss, loss, accumulate);
 }
 
 cudaError_t launch_loss_accum(const double* loss_part, int n, double* acc, int accumulate, cudaStream_t st) {
-  k_loss_accum<<<1, 256, 0, st>>>(loss_part, n, acc, accumulate);
-  return cudaGetLastError();
+  return launch_after(k_loss_accum, 1, 256, 0, st, loss_part, n, acc, accumulate);
 }
 
 cudaError_t launch_update(const UpdateArgs& u, cudaStream_t st) {
@@ -459,11 +469,7 @@ cudaError_t launch_update(const UpdateArgs& u, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const size_t blocks = (n + 255) / 256;
   const unsigned grid = (unsigned)(blocks < 4096 ? blocks : 4096);
-  if (u.acc)
-    k_update<true><<<grid, 256, 0, st>>>(u);
-  else
-    k_update<false><<<grid, 256, 0, st>>>(u);
-  return cudaGetLastError();
+  return launch_after(u.acc ? k_update<true> : k_update<false>, grid, 256, 0, st, u);
 }
 
 cudaError_t launch_norm2(const float2* x, size_t n, double* part, int n_part, double* out, int slot,
