@@ -282,7 +282,7 @@ __device__ __forceinline__ void gm_store_loss(double lsum, double* red, double* 
 // gradient (the object-gradient accumulation skips such windows).
 template <int KIND>
 __device__ __forceinline__ void gm_skip(const GmBlock& b, int L, int parts, int part, int t, int T) {
-  if (KIND == GM_FWD && t == 0) *b.a.status = PTYCHO_ERR_POSITION;
+  if (KIND == GM_FWD && t == 0) *b.a.pos_status = PTYCHO_ERR_POSITION;
   if (KIND == GM_RES && t == 0 && b.g.mode != MODE_FORWARD) b.a.loss_part[(size_t)b.il * parts + part] = 0.0;
   if (KIND == GM_ADJ && b.g.s == 0)
     for (int k = t; k < L * b.M; k += T) b.g.dst[(size_t)b.il * b.M * b.M + b.at(k % L, k / L)] = make_float2(0.f, 0.f);

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_chain_tc(const ChainArgs a, c
   const int yi = r.x, xi = r.y;
   if (yi < 0 || xi < 0 || yi > a.H - TM || xi > a.W - TM) {
     if (t == 0) {
-      *a.status = PTYCHO_ERR_POSITION;
+      *a.pos_status = PTYCHO_ERR_POSITION;
       if (MODE != MODE_FORWARD) a.loss_part[il] = 0.0;
     }
     if (MODE == MODE_GRAD)

@@ -68,7 +68,9 @@ struct ChainArgs {
   double* loss_part;      // [n_pos] (generic windows: [n_pos][gm_loss_parts(M)])
   float2* psi_out;        // [N][M][M] or null (forward mode)
   float* int_out;         // [N][M][M] or null (forward mode)
-  int* status;            // device error word (PTYCHO_ERR_POSITION on a bad window)
+  int* status;            // device error word
+  int* pos_status;        // where a window outside the object is flagged (PTYCHO_ERR_POSITION):
+                          // the error word, or a word nobody reads when the host checks
   int selftest_timeout;   // PTYCHO_FLAG_SELFTEST_TIMEOUT: the split-product kernel issues no MMAs
 };
 

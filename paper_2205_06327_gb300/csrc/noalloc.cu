@@ -191,6 +191,7 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
   a.ws_gp = ws_gp;
   a.loss_part = loss_part;
   a.status = d_status;
+  a.pos_status = d_status;
   const bool want_grad = grad_obj || grad_probe;
   for (int c0 = 0, ci = 0; c0 < p.N; c0 += chunk, ++ci) {
     const int n = p.N - c0 < chunk ? p.N - c0 : chunk;

@@ -189,7 +189,8 @@ struct ptycho_plan_s {
   int loss_parts = 1;           // loss parts per position (generic-window path: its line blocks)
   double* d_scal = nullptr;   // [8]: 0 loss, 1 |gO|^2, 2 |gP|^2, 3 trial loss
   double* norm_part = nullptr;  // [kNormParts]
-  int* d_status = nullptr;
+  int* d_status = nullptr;    // [2]: the error word, and the word of host-checked plans' chains
+  cudaEvent_t ev_check = nullptr;  // the positions have reached h_pos
   int* h_pos = nullptr;       // pinned, [N][2]
   double* h_scal = nullptr;   // pinned, [8]
   int* h_flag = nullptr;      // pinned, [1]: the device error word, read by the synchronous calls
@@ -246,6 +247,7 @@ void free_plan(ptycho_plan pl) {
   cudaFree(pl->g_obj);
   cudaFree(pl->g_probe);
   cudaFree(pl->d_cplanes);
+  if (pl->ev_check) cudaEventDestroy(pl->ev_check);
   if (pl->ev_fork) cudaEventDestroy(pl->ev_fork);
   if (pl->ev_join) cudaEventDestroy(pl->ev_join);
   if (pl->side) cudaStreamDestroy(pl->side);
@@ -315,16 +317,30 @@ int status_fail(int h) {
 }
 
 // Positions check on the host (pinned copy) unless the plan asks for the
-// asynchronous device-side check only.
-int check_positions(ptycho_plan pl, const int32_t* pos, cudaStream_t st) {
+// asynchronous device-side check only.  It comes in two halves so that the
+// chain, which skips bad windows by itself and writes only the workspace, can
+// be launched between them and run while the copy is waited for (64 positions,
+// M = 64, one slice: 60 -> 52 us a call).
+int begin_check(ptycho_plan pl, const int32_t* pos, cudaStream_t st) {
   const ptycho_params& p = pl->p;
   if (p.N == 0) return PTYCHO_OK;
   if (!is_device_ptr(pos)) return fail(PTYCHO_ERR_ARG, "pos_yx must be a device pointer");
   if (!aligned(pos, 8)) return fail(PTYCHO_ERR_ARG, "pos_yx must be 8-byte aligned");
   if (p.flags & PTYCHO_FLAG_ASYNC_CHECK) return PTYCHO_OK;
   CUDA_TRY(cudaMemcpyAsync(pl->h_pos, pos, sizeof(int32_t) * 2 * (size_t)p.N, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaStreamSynchronize(st));
-  return check_windows(p, pl->h_pos);
+  CUDA_TRY(cudaEventRecord(pl->ev_check, st));
+  return PTYCHO_OK;
+}
+
+int end_check(ptycho_plan pl) {
+  if (pl->p.N == 0 || (pl->p.flags & PTYCHO_FLAG_ASYNC_CHECK)) return PTYCHO_OK;
+  CUDA_TRY(cudaEventSynchronize(pl->ev_check));
+  return check_windows(pl->p, pl->h_pos);
+}
+
+int check_positions(ptycho_plan pl, const int32_t* pos, cudaStream_t st) {
+  const int rc = begin_check(pl, pos, st);
+  return rc ? rc : end_check(pl);
 }
 
 // Every window inside the object: 0 <= y <= H - M, 0 <= x <= W - M.
@@ -402,6 +418,7 @@ ChainArgs base_args(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe,
   a.ws_gp = pl->ws_gp;
   a.loss_part = pl->loss_part;
   a.status = pl->d_status;
+  a.pos_status = pl->d_status + (pl->p.flags & PTYCHO_FLAG_ASYNC_CHECK ? 0 : 1);
   a.selftest_timeout = (pl->p.flags & PTYCHO_FLAG_SELFTEST_TIMEOUT) ? 1 : 0;
   return a;
 }
@@ -466,7 +483,7 @@ int update_step(ptycho_plan pl, ptycho_c64* obj, ptycho_c64* probe, double a_o, 
 int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, const ptycho_c64* obj,
                   const float* meas, float2* grad_obj, float2* grad_probe, int slot, const float2* obj_dir,
                   float obj_step, const float2* probe_dir, float probe_step, cudaStream_t st,
-                  int n_first = 0, cudaEvent_t rest_ready = nullptr) {
+                  int n_first = 0, cudaEvent_t rest_ready = nullptr, bool check = false) {
   const ptycho_params& p = pl->p;
   const bool want_grad = grad_obj || grad_probe;
   if (p.N == 0) {
@@ -565,6 +582,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
     } else if ((rc = launch_chain_for(a)) != PTYCHO_OK) {
       return rc;
     }
+    if (check && ci == 0 && (rc = end_check(pl)) != PTYCHO_OK) return rc;
     if (recompute) {
       // The first launch differentiated the last segment; each later one
       // rebuilds and differentiates the segment before it, whose patches
@@ -731,12 +749,14 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
   if (!rc) rc = dev_alloc(&pl->loss_part, (size_t)pl->chunk * pl->loss_parts, "loss partials");
   if (!rc) rc = dev_alloc(&pl->d_scal, 8, "scalars");
   if (!rc) rc = dev_alloc(&pl->norm_part, kNormParts, "norm partials");
-  if (!rc) rc = dev_alloc(&pl->d_status, 1, "status");
+  if (!rc) rc = dev_alloc(&pl->d_status, 2, "status");
   std::vector<uint32_t> planes;
   if (!rc && p.precision != PTYCHO_FP32) {
     planes = build_tc_planes(p, p.precision == PTYCHO_FP16X3);
     rc = dev_alloc(&pl->d_cplanes, planes.size(), "tensor-core operand planes");
   }
+  if (!rc && (e = cudaEventCreateWithFlags(&pl->ev_check, cudaEventDisableTiming)) != cudaSuccess)
+    rc = cuda_fail(e, "check event");
   if (!rc && !gm &&
       ((e = cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking)) != cudaSuccess ||
        (e = cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
@@ -764,7 +784,7 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
       (e = cudaMemcpy(pl->d_hs, hs.data(), M * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (!h2.empty() &&
        (e = cudaMemcpy(pl->d_h2, h2.data(), h2.size() * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (e = cudaMemset(pl->d_status, 0, sizeof(int))) != cudaSuccess ||
+      (e = cudaMemset(pl->d_status, 0, 2 * sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(pl->d_scal, 0, 8 * sizeof(double))) != cudaSuccess) {
     free_plan(pl);
     return cuda_fail(e, "table upload");
@@ -868,9 +888,9 @@ int loss_grad_impl(ptycho_plan plan, const int32_t* pos_yx, const ptycho_c64* pr
       (rc = check_array(meas_I, "meas_I", plan->p.N > 0)) || (rc = check_array(grad_obj, "grad_obj", false)) ||
       (rc = check_array(grad_probe, "grad_probe", false)))
     return rc;
-  if ((rc = check_positions(plan, pos_yx, st))) return rc;
+  if ((rc = begin_check(plan, pos_yx, st))) return rc;
   rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, reinterpret_cast<float2*>(grad_obj),
-                     reinterpret_cast<float2*>(grad_probe), 0, nullptr, 0.f, nullptr, 0.f, st);
+                     reinterpret_cast<float2*>(grad_probe), 0, nullptr, 0.f, nullptr, 0.f, st, 0, nullptr, true);
   if (rc) return rc;
   return deliver_loss(plan, 0, loss_out, st);
 }
@@ -886,11 +906,12 @@ int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho
   if ((rc = check_array(probe, "probe", true)) || (rc = check_array(obj, "obj", true)) ||
       (rc = check_array(meas_I, "meas_I", p.N > 0)))
     return rc;
-  if ((rc = check_positions(plan, pos_yx, st))) return rc;
+  if ((rc = begin_check(plan, pos_yx, st))) return rc;
   const size_t nO = (size_t)p.S * p.H * p.W, nP = (size_t)p.M * p.M;
   if (!plan->g_obj && (rc = dev_alloc(&plan->g_obj, nO, "step object gradient"))) return rc;
   if (!plan->g_probe && (rc = dev_alloc(&plan->g_probe, nP, "step probe gradient"))) return rc;
-  rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, plan->g_obj, plan->g_probe, 0, nullptr, 0.f, nullptr, 0.f, st);
+  rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, plan->g_obj, plan->g_probe, 0, nullptr, 0.f, nullptr, 0.f, st,
+                     0, nullptr, true);
   if (rc) return rc;
   if ((rc = deliver_loss(plan, 0, loss_out, st))) return rc;
   ptycho_plan pl = plan;
