@@ -344,6 +344,38 @@ cudaError_t gm_prepare(int M) {
   return cudaFuncSetAttribute(k_gm_pass_rt<GM_RES>, attr, (int)most);
 }
 
+// Positions per chunk for n positions, at most cap.  A pass runs in waves of
+// resident blocks; a chunk that ends in a nearly empty wave, or a small last
+// chunk, wastes them in each of its 2S + 1 passes.  Takes the chunk with the
+// fewest waves in all, a fifth of a wave counted per chunk for its launches.
+// us of an evaluation, largest chunk / this rule: 506 positions, M = 192 3107 /
+// 3068; 306 simulated at 256 791 / 777; 400, M = 81 420 / 413; 1024, M = 256
+// 7445 / 7483.
+int gm_chunk(int M, int n, int cap, int sm_count) {
+  if (n <= cap) return n;
+  const GmInstance* in = gm_find(M);
+  int per_sm = 0;
+  if (in)
+    per_sm = in->blocks_per_sm();
+  else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gm_pass_rt<GM_ADJ>, kGmThreads, gm_rt_smem(M)) !=
+           cudaSuccess)
+    per_sm = 0;
+  const double resident = (double)per_sm * sm_count;
+  if (resident <= 0) return cap;
+  const int parts = gm_loss_parts(M);
+  auto waves = [&](int positions) { return std::ceil(positions * (double)parts / resident) + 0.2; };
+  int best = cap;
+  double least = 0;
+  for (int c = cap; c >= 1 && 2 * c >= cap; --c) {
+    const double w = n / c * waves(c) + (n % c ? waves(n % c) : 0);
+    if (c == cap || w < least) {
+      best = c;
+      least = w;
+    }
+  }
+  return best;
+}
+
 namespace {
 
 struct GmLauncher {

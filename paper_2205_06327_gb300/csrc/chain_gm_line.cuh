@@ -44,6 +44,7 @@ struct GmInstance {
   int r1, r2, r3;
   int parts;  // loss parts per position (blocks of the residual pass)
   cudaError_t (*prepare)();
+  int (*blocks_per_sm)();  // resident blocks of a pass (0 if unknown)
   cudaError_t (*launch)(GmKind kind, const ChainArgs& a, const GmPass& g, cudaStream_t st);
 };
 
@@ -596,8 +597,16 @@ cudaError_t gm_launch_ct(GmKind kind, const ChainArgs& a, const GmPass& g, cudaS
 }
 
 template <class P>
+int gm_blocks_ct() {
+  int n = 0;
+  const cudaError_t e =
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gm_pass<P, GM_ADJ, false>, P::T, P::smem(false));
+  return e == cudaSuccess ? n : 0;
+}
+
+template <class P>
 constexpr GmInstance gm_instance() {
-  return GmInstance{P::M, P::R1, P::R2, P::R3, P::M / P::L, gm_prepare_ct<P>, gm_launch_ct<P>};
+  return GmInstance{P::M, P::R1, P::R2, P::R3, P::M / P::L, gm_prepare_ct<P>, gm_blocks_ct<P>, gm_launch_ct<P>};
 }
 
 }  // namespace

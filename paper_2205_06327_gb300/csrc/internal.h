@@ -105,6 +105,7 @@ bool gm_supported(int M);
 void gm_factor_gain(int M, double* gain);
 int gm_loss_parts(int M);  // loss parts the chain writes per position
 cudaError_t gm_prepare(int M);
+int gm_chunk(int M, int n, int cap, int sm_count);  // after gm_prepare
 cudaError_t launch_chain_gm(ChainMode mode, const ChainArgs& a, float2* wv, int M, int* n_launches,
                             cudaStream_t st);
 

@@ -162,9 +162,7 @@ std::vector<uint32_t> build_tc_planes(const ptycho_params& p, bool f16) {
 
 constexpr int64_t kDefaultWorkspace = 8ll << 30;
 // Generic-window path: the most bytes of chunk waves (streamed by every pass)
-#ifndef PTYCHO_GM_WAVE_BYTES
-#define PTYCHO_GM_WAVE_BYTES (64ll << 20)
-#endif
+constexpr int64_t kGmWaveBytes = 64ll << 20;
 constexpr int kProbeSplit = 32;
 constexpr int kNormParts = 512;
 
@@ -714,10 +712,15 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
       (psi_slots + gphi_slots + (gm ? 1 : 0)) * MM * sizeof(float2) + MM * sizeof(float2) + sizeof(double);
   const int64_t cap = p.workspace_bytes ? p.workspace_bytes : kDefaultWorkspace;
   int64_t chunk = cap / (int64_t)per_pos;
-  // generic-window path: keep the chunk's waves (streamed by every FFT pass)
-  // within about half of the L2
+  // generic-window path: keep the chunk's waves (streamed by every pass) within
+  // about half of the L2, or three quarters where that saves splitting the
+  // positions (930 at M = 96, 68 MB: 1480 us in two chunks, 1389 in one; 196 at
+  // M = 216, 73 MB: 1854, 1762; several chunks of up to 96 MB: 506 at M = 192
+  // 3068, 3100, 1024 at M = 256 7482, 7633)
   if (gm && chunk > 1) {
-    const int64_t l2cap = (int64_t)PTYCHO_GM_WAVE_BYTES / (int64_t)(MM * sizeof(float2));
+    const int64_t wave = (int64_t)(MM * sizeof(float2));
+    const bool whole = M < 256 && p.N * wave <= kGmWaveBytes / 2 * 3;
+    const int64_t l2cap = whole ? p.N : kGmWaveBytes / wave;
     if (chunk > l2cap) chunk = l2cap > 1 ? l2cap : 1;
   }
   if (chunk < 1) {
@@ -727,6 +730,8 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
   const int n = p.N > 0 ? p.N : 1;
   if (chunk >= n) {
     chunk = n;
+  } else if (gm) {
+    chunk = gm_chunk(M, n, (int)chunk, pl->sm_count);
   } else {
     const int blocks_per_wave = pl->sm_count * (M == 128 ? 1 : 4);
     if (chunk > blocks_per_wave) chunk -= chunk % blocks_per_wave;
