@@ -948,12 +948,7 @@ int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho
   return PTYCHO_OK;
 }
 
-// Run fn(problem) for every problem, in order, on st.  (Running the problems
-// concurrently on their own streams was measured slower on the batched
-// workload: the generic-window problems size their chunks to the L2 and then
-// compete for it.)  Returns the first error, tagged with the problem's index.
-template <class F>
-int run_multi(const ptycho_problem* probs, int32_t n, F&& fn) {
+int check_problems(const ptycho_problem* probs, int32_t n) {
   if (n < 0 || (n > 0 && !probs)) return fail(PTYCHO_ERR_ARG, "problems must be non-NULL and n >= 0");
   for (int32_t i = 0; i < n; ++i) {
     if (!probs[i].plan) return fail(PTYCHO_ERR_ARG, "problem " + std::to_string(i) + ": plan is NULL");
@@ -963,13 +958,6 @@ int run_multi(const ptycho_problem* probs, int32_t n, F&& fn) {
       if (probs[j].plan == probs[i].plan)
         return fail(PTYCHO_ERR_ARG, "problems " + std::to_string(j) + " and " + std::to_string(i) +
                                         " share a plan");
-  }
-  for (int32_t i = 0; i < n; ++i) {
-    const int rc = fn(probs[i]);
-    if (rc) {
-      g_last_error = "problem " + std::to_string(i) + ": " + g_last_error;
-      return rc;
-    }
   }
   return PTYCHO_OK;
 }
@@ -1071,6 +1059,39 @@ int run_multi_fused(const ptycho_problem* probs, const std::vector<int>& idx, bo
     if (step && (rc = update_step(pl, q.obj, q.probe, -a_o, -a_p, nullptr, 0, st))) return rc;
   }
   return PTYCHO_OK;
+}
+
+// The problems of one call: those in `fused` through run_multi_fused, the
+// others through fn(problem), in order, on st.  With both kinds present the
+// fused ones run on a side stream forked from st and joined back: their chains
+// keep their waves on chip, so they fill the SMs that the line passes' partial
+// waves leave idle without competing for the L2 (one problem per window class,
+// 1428 positions, graph replay: 3171 -> 3049 us).  Each kind by itself stays on one
+// stream: the line passes size their chunks to the L2.
+template <class F>
+int run_multi(const ptycho_problem* probs, int32_t n, const std::vector<int>& fused, bool step, double a_o, double a_p,
+              cudaStream_t st, F&& fn) {
+  const bool fork = !fused.empty() && (int32_t)fused.size() < n;
+  ptycho_plan fp = fork ? probs[fused[0]].plan : nullptr;
+  cudaStream_t fst = st;
+  if (fork) {
+    fst = fp->side;
+    CUDA_TRY(cudaEventRecord(fp->ev_fork, st));
+    CUDA_TRY(cudaStreamWaitEvent(fst, fp->ev_fork, 0));
+  }
+  int rc = run_multi_fused(probs, fused, step, a_o, a_p, fst);
+  for (int32_t i = 0, k = 0; !rc && i < n; ++i) {
+    if (k < (int32_t)fused.size() && fused[k] == i) {
+      ++k;
+      continue;
+    }
+    if ((rc = fn(probs[i]))) g_last_error = "problem " + std::to_string(i) + ": " + g_last_error;
+  }
+  if (fork) {
+    CUDA_TRY(cudaEventRecord(fp->ev_join, fst));
+    CUDA_TRY(cudaStreamWaitEvent(st, fp->ev_join, 0));
+  }
+  return rc;
 }
 
 // ptycho_loss_grad_host: host arrays in and out.  The inputs are staged in
@@ -1207,15 +1228,14 @@ int ptycho_step_accumulate(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* 
 int ptycho_multi_loss_grad(const ptycho_problem* problems, int32_t n, void* stream) {
   g_last_error.clear();
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  int rc = check_problems(problems, n);
+  if (rc) return rc;
   std::vector<int> fused;
-  int rc = run_multi(problems, n, [&](const ptycho_problem& q) {
-    if (fusable(q.plan) && (q.grad_obj || q.grad_probe)) {  // loss-only problems take the cheaper chain
-      fused.push_back((int)(&q - problems));
-      return PTYCHO_OK;
-    }
+  for (int32_t i = 0; i < n; ++i)  // loss-only problems take the cheaper chain
+    if (fusable(problems[i].plan) && (problems[i].grad_obj || problems[i].grad_probe)) fused.push_back(i);
+  return run_multi(problems, n, fused, false, 0.0, 0.0, st, [&](const ptycho_problem& q) {
     return loss_grad_impl(q.plan, q.pos_yx, q.probe, q.obj, q.meas_I, q.loss_out, q.grad_obj, q.grad_probe, st);
   });
-  return rc ? rc : run_multi_fused(problems, fused, false, 0.0, 0.0, st);
 }
 
 int ptycho_multi_step(const ptycho_problem* problems, int32_t n, double alpha_obj, double alpha_probe,
@@ -1224,16 +1244,14 @@ int ptycho_multi_step(const ptycho_problem* problems, int32_t n, double alpha_ob
   if (!std::isfinite(alpha_obj) || !std::isfinite(alpha_probe))
     return fail(PTYCHO_ERR_ARG, "step sizes must be finite");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  int rc = check_problems(problems, n);
+  if (rc) return rc;
   std::vector<int> fused;
-  int rc = run_multi(problems, n, [&](const ptycho_problem& q) {
-    if (fusable(q.plan)) {
-      fused.push_back((int)(&q - problems));
-      return PTYCHO_OK;
-    }
-    return step_impl(q.plan, q.pos_yx, q.probe, q.obj, q.meas_I, alpha_obj, alpha_probe, 0, q.loss_out, nullptr,
-                     st);
+  for (int32_t i = 0; i < n; ++i)
+    if (fusable(problems[i].plan)) fused.push_back(i);
+  return run_multi(problems, n, fused, true, alpha_obj, alpha_probe, st, [&](const ptycho_problem& q) {
+    return step_impl(q.plan, q.pos_yx, q.probe, q.obj, q.meas_I, alpha_obj, alpha_probe, 0, q.loss_out, nullptr, st);
   });
-  return rc ? rc : run_multi_fused(problems, fused, true, alpha_obj, alpha_probe, st);
 }
 
 int ptycho_potential_to_transmission(const float* V, ptycho_c64* obj, int64_t n, double sigma, void* stream) {
