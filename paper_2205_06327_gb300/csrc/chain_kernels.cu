@@ -98,7 +98,7 @@ __device__ __forceinline__ void store_patch(float2* p, float2 v) {
 
 template <int M, int MODE>
 __global__ void __launch_bounds__(Cfg<M>::T, Cfg<M>::MIN_BLOCKS) k_chain(const ChainArgs a) {
-  using C = Cfg<M>;
+  using C = std::conditional_t<MODE == MODE_FORWARD || MODE == MODE_LOSS, HalfFetch<Cfg<M>>, Cfg<M>>;
   const int il = blockIdx.x, t = threadIdx.x;
 #include "chain_body.inc"
 }

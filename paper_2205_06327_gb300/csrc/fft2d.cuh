@@ -201,6 +201,7 @@ template <>
 struct Cfg<128> {
   static constexpr int M = 128, T = 512, V = 32, MIN_BLOCKS = 1;
   static constexpr int CL = 1, TB = T, kSmemWave = M * M;  // blocks per position, threads per block
+  static constexpr int TWB = 16;  // complex factors fetched from tensor memory at a time
   __device__ static __forceinline__ void sync() { __syncthreads(); }
   __device__ static __forceinline__ void arrived(const Factors&, int) { __syncthreads(); }
   __device__ static __forceinline__ void put_loss(double* red, int w, double v) { red[w] = v; }
@@ -298,7 +299,7 @@ struct ClusterCfg128 : Cfg<128> {
 template <>
 struct Cfg<64> {
   static constexpr int M = 64, T = 128, V = 32, MIN_BLOCKS = 4;
-  static constexpr int CL = 1, TB = T, kSmemWave = M * M;
+  static constexpr int CL = 1, TB = T, kSmemWave = M * M, TWB = 16;
   __device__ static __forceinline__ void sync() { __syncthreads(); }
   __device__ static __forceinline__ void arrived(const Factors&, int) { __syncthreads(); }
   __device__ static __forceinline__ void put_loss(double* red, int w, double v) { red[w] = v; }
@@ -325,6 +326,15 @@ struct Cfg<64> {
       py = 16 * w + 4 * d2; px = 16 * e1 + 4 * e2;
     }
   }
+};
+
+// The same with half the factors fetched at a time.  Fewer, wider fetches wait
+// less but hold more registers: 576 positions, M = 128, 16 slices, gradient
+// 1606 us with 8 at a time, 1587 with 16 (4560 positions in recompute mode 27.3
+// and 26.9 ms); forward model alone 538 and 554 us.
+template <class B>
+struct HalfFetch : B {
+  static constexpr int TWB = 8;
 };
 
 // Frequency index of storage row/column after the three forward passes:
@@ -425,6 +435,22 @@ __device__ __forceinline__ void tmem_factors8(uint32_t taddr, float2 (&w)[8]) {
   for (int i = 0; i < 8; ++i) w[i] = make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
 }
 
+// 16 of them.
+__device__ __forceinline__ void tmem_factors16(uint32_t taddr, float2 (&w)[16]) {
+  float2* p = w;
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\ttcgen05.wait::ld.sync.aligned;"
+      : "=f"(p[0].x), "=f"(p[0].y), "=f"(p[1].x), "=f"(p[1].y), "=f"(p[2].x), "=f"(p[2].y), "=f"(p[3].x),
+        "=f"(p[3].y), "=f"(p[4].x), "=f"(p[4].y), "=f"(p[5].x), "=f"(p[5].y), "=f"(p[6].x), "=f"(p[6].y),
+        "=f"(p[7].x), "=f"(p[7].y), "=f"(p[8].x), "=f"(p[8].y), "=f"(p[9].x), "=f"(p[9].y), "=f"(p[10].x),
+        "=f"(p[10].y), "=f"(p[11].x), "=f"(p[11].y), "=f"(p[12].x), "=f"(p[12].y), "=f"(p[13].x), "=f"(p[13].y),
+        "=f"(p[14].x), "=f"(p[14].y), "=f"(p[15].x), "=f"(p[15].y)
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_factors(uint32_t a, float2 (&w)[8]) { tmem_factors8(a, w); }
+__device__ __forceinline__ void tmem_factors(uint32_t a, float2 (&w)[16]) { tmem_factors16(a, w); }
+
 // All V complex values of the thread's tensor-memory words [word, word + 2V):
 // issued here, usable after tmem_factors_wait.
 __device__ __forceinline__ void tmem_factors_issue(uint32_t taddr, float2 (&w)[32]) {
@@ -490,13 +516,13 @@ __device__ __forceinline__ void pass_compute(float2 (&v)[C::V], const Factors& f
   t = opaque(t);
   auto twiddle = [&]() {
     if constexpr (J == 0) {
-      static_for<0, C::V / 8>([&](auto cc) {
+      static_for<0, C::V / C::TWB>([&](auto cc) {
         constexpr int c = decltype(cc)::value;
-        float2 w[8];
-        tmem_factors8(f.tmem + 16 * c, w);
-        static_for<0, 8>([&](auto ii) {
-          constexpr int e = 8 * c + decltype(ii)::value;
-          if constexpr (e % P::G != 0) v[e] = pmul_opt<INV>(v[e], w[e % 8]);
+        float2 w[C::TWB];
+        tmem_factors(f.tmem + 2 * C::TWB * c, w);
+        static_for<0, C::TWB>([&](auto ii) {
+          constexpr int e = C::TWB * c + decltype(ii)::value;
+          if constexpr (e % P::G != 0) v[e] = pmul_opt<INV>(v[e], w[e % C::TWB]);
         });
       });
     } else if constexpr (J == 1) {
@@ -585,13 +611,13 @@ __device__ __forceinline__ void mul_prop(float2 (&v)[C::V], const Factors& f) {
     mul_factors<CONJ, 1>(v, w);
     return;
   }
-  static_for<0, C::V / 8>([&](auto cc) {
+  static_for<0, C::V / C::TWB>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
-    float2 w[8];
-    tmem_factors8(f.tmem + 2 * C::V + 16 * c, w);
-    static_for<0, 8>([&](auto ii) {
-      constexpr int e = 8 * c + decltype(ii)::value;
-      v[e] = pmul_opt<CONJ>(v[e], w[e % 8]);
+    float2 w[C::TWB];
+    tmem_factors(f.tmem + 2 * C::V + 2 * C::TWB * c, w);
+    static_for<0, C::TWB>([&](auto ii) {
+      constexpr int e = C::TWB * c + decltype(ii)::value;
+      v[e] = pmul_opt<CONJ>(v[e], w[e % C::TWB]);
     });
   });
 }
