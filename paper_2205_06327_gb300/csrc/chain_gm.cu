@@ -306,19 +306,21 @@ void gm_factor_gain(int M, double* gain) {
       f1[k] += D1[(size_t)k * R1 + n] * tone / (double)R1;
       i1[k] += std::conj(D1[(size_t)n * R1 + k] * tone) / (double)R1;
     }
+  std::vector<cd> w(M), wr(M);  // exp(-2 pi i e / M), exact and rounded
+  for (int e = 0; e < M; ++e) wr[e] = rounded(w[e] = root(M, e));
   for (int k = 0; k < M; ++k) {
     const int k1 = k % R1, kap = k / R1, k2 = kap % R2, k3 = kap / R2;
     cd f = 0, b = 0;
     for (int j = 0; j < MI; ++j) {
       const int j2 = j % R3, q2 = j / R3;
-      const cd tone = std::conj(root(MI, kap * j));
-      // twiddles of both splits, each as (rounded / exact)
-      cd tw = rounded(root(M, k1 * j)) / root(M, k1 * j);
-      const cd t2 = R2 > 1 ? rounded(root(MI, k2 * j2)) : cd(1);
-      f += D2[(size_t)k2 * R2 + q2] * t2 * D3[(size_t)k3 * R3 + j2] * tone * tw / (double)MI;
-      b += std::conj(D2[(size_t)q2 * R2 + k2] * t2 * D3[(size_t)j2 * R3 + k3] * tone * tw) / (double)MI;
+      // the tone, with the first split's twiddle as rounded / exact, and the
+      // second split's twiddle
+      cd u = std::conj(w[R1 * (kap * j % MI)]) * wr[k1 * j] * std::conj(w[k1 * j]);
+      if (R2 > 1) u *= wr[R1 * k2 * j2];
+      f += D2[(size_t)k2 * R2 + q2] * D3[(size_t)k3 * R3 + j2] * u;
+      b += std::conj(D2[(size_t)q2 * R2 + k2] * D3[(size_t)j2 * R3 + k3] * u);
     }
-    gain[k] = std::abs(f1[k1] * i1[k1] * f * b);
+    gain[k] = std::abs(f1[k1] * i1[k1] * f * b) / ((double)MI * MI);
   }
 }
 
