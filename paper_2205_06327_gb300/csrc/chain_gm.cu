@@ -183,12 +183,15 @@ __global__ void __launch_bounds__(kGmThreads, 4)
     transform(std::false_type{});
     double lsum = 0.0;
     const size_t e0 = (size_t)(a.pos_begin + il) * M * M;
+    if (g.mode == MODE_FORWARD) {
+      each([&](int li, int i) { gm_output(b, x[li * LS + gm_pad(i)], e0 + b.at(li, i)); });
+      return;
+    }
     each([&](int li, int i) {
       float2& v = x[li * LS + gm_pad(i)];
-      v = gm_residual(b, v, e0 + b.at(li, i), lsum);
+      v = gm_residual(M, v, __ldcs(a.meas + e0 + b.at(li, i)), lsum);
     });
-    if (g.mode != MODE_FORWARD)
-      gm_store_loss<kGmThreads>(lsum, red, a.loss_part + (size_t)il * parts + part, t);
+    gm_store_loss<kGmThreads>(lsum, red, a.loss_part + (size_t)il * parts + part, t);
     if (!g.dst) return;
     __syncthreads();
     transform(std::true_type{});

@@ -246,22 +246,24 @@ struct GmBlock {
   }
 };
 
-// Far field (unnormalised along both axes: M Psi) -> outputs (forward mode)
-// or the residual of Eq. 1: adds the loss terms to lsum and returns the
-// adjoint seed 2 d Psi/|Psi| / M, pre-scaled for the unnormalised inverse.
-__device__ __forceinline__ float2 gm_residual(const GmBlock& b, float2 z, size_t e, double& lsum) {
+// Far field z (unnormalised along both axes: M Psi) of element e -> outputs
+// (forward mode).
+__device__ __forceinline__ void gm_output(const GmBlock& b, float2 z, size_t e) {
   const float inv_m = 1.0f / (float)b.M;
-  if (b.g.mode == MODE_FORWARD) {
-    const float2 p = make_float2(z.x * inv_m, z.y * inv_m);
-    if (b.a.psi_out) b.a.psi_out[e] = p;
-    if (b.a.int_out) b.a.int_out[e] = fmaf(p.x, p.x, p.y * p.y);
-    return p;
-  }
-  const float A = sqrtf(__ldg(b.a.meas + e));
+  const float2 p = make_float2(z.x * inv_m, z.y * inv_m);
+  if (b.a.psi_out) b.a.psi_out[e] = p;
+  if (b.a.int_out) b.a.int_out[e] = fmaf(p.x, p.x, p.y * p.y);
+}
+
+// The residual of Eq. 1 against the measured intensity: adds the loss term to
+// lsum and returns the adjoint seed 2 d Psi/|Psi| / M, pre-scaled for the
+// unnormalised inverse.
+__device__ __forceinline__ float2 gm_residual(int M, float2 z, float intensity, double& lsum) {
+  const float A = sqrtf(intensity);
   const float mag = sqrtf(fmaf(z.x, z.x, z.y * z.y));
-  const float d = mag * inv_m - A;
+  const float d = mag * (1.0f / (float)M) - A;
   lsum += (double)d * (double)d;
-  const float sc = mag > 0.0f ? (2.0f * d) / (mag * (float)b.M) : 0.0f;
+  const float sc = mag > 0.0f ? (2.0f * d) / (mag * (float)M) : 0.0f;
   return make_float2(z.x * sc, z.y * sc);
 }
 
@@ -495,15 +497,27 @@ __global__ void __launch_bounds__(P::T, P::MINB) k_gm_pass(const ChainArgs a, co
     ln.template phase_b<false>();
     double lsum = 0.0;
     const size_t e0 = (size_t)(a.pos_begin + il) * M * M;
+    if (g.mode == MODE_FORWARD) {
+      ln.template items<R1 * R2>([&](int li, int r) {
+        float2 x[R3];
+        ln.get_c(x, li, r % R1, r / R1);
+#pragma unroll
+        for (int q = 0; q < R3; ++q) gm_output(b, x[q], e0 + b.at(li, r + R1 * R2 * q));
+      });
+      return;
+    }
     ln.template items<R1 * R2>([&](int li, int r) {
       const int k1 = r % R1, k2 = r / R1;
+      float I[R3];  // from DRAM: fetched before the transform
+#pragma unroll
+      for (int q = 0; q < R3; ++q) I[q] = __ldcs(a.meas + e0 + b.at(li, r + R1 * R2 * q));
       float2 x[R3];
       ln.get_c(x, li, k1, k2);
 #pragma unroll
-      for (int q = 0; q < R3; ++q) x[q] = gm_residual(b, x[q], e0 + b.at(li, r + R1 * R2 * q), lsum);
+      for (int q = 0; q < R3; ++q) x[q] = gm_residual(M, x[q], I[q], lsum);
       if (g.dst) ln.put_c(x, li, k1, k2);
     });
-    if (g.mode != MODE_FORWARD) gm_store_loss<T>(lsum, red, a.loss_part + (size_t)il * PARTS + part, t);
+    gm_store_loss<T>(lsum, red, a.loss_part + (size_t)il * PARTS + part, t);
     if (!g.dst) return;
     ln.sync();
     ln.template phase_b<true>();
