@@ -46,8 +46,8 @@ struct AccVec<1> {
 // tile: the row's sums live in shared memory and only that warp touches them.
 // The warp walks the positions whose window covers its row in ascending order
 // and streams that window row of psi and g_phi, VEC pixels per lane and step
-// (16-byte loads for even windows), K steps per position, with the loads of U
-// positions in flight before the first is added.
+// (16-byte loads for even windows), K steps per position, with the loads of
+// groups of U positions in flight before they are added.
 //
 // The kernel is bound by HBM: it reads the two workspace arrays once.  With
 // threads tied to the pixels of a 32 x 32 tile, a third of the loads fell
@@ -75,7 +75,19 @@ template <int K, int VEC, bool PATCH>
 __global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumArgs a) {
   using V = AccVec<VEC>;
   using vec = typename V::type;
-  constexpr int STEPS = PATCH ? 16 : 8, U = STEPS / K;
+  // Two groups of loads in turn, one in flight while the other is added, or one
+  // twice as large.  ncu on the latter (patches, M = 128): waiting for loads is
+  // half of all stalls at 4 TB/s.  One group / two: 4560 patches of 30 slices,
+  // M = 128 (K = 2) 4.49 / 3.20 ms, M = 64 (K = 1) 0.93 / 1.06 ms; waves of 930
+  // positions, M = 96 (K = 2) 311 / 274 us, 576 at 128 606 / 593, 225 at 192 (K =
+  // 3) 235 / 234, 4 at 1024 (K = 8) 81 / 111.
+  constexpr bool PIPE = PATCH ? K >= 2 : K <= 3;
+  constexpr int STEPS = PIPE ? (PATCH ? 8 : 4) : (PATCH ? 16 : 8), U = STEPS / K > 0 ? STEPS / K : 1;
+  struct Group {  // positions whose loads are in flight together
+    vec g[U][K];
+    vec p[PATCH ? 1 : U][PATCH ? 1 : K];
+    int cx[U], lo[U], hi[U];  // tile column of window column 0; window columns [lo, hi) of the segment
+  };
   __shared__ int2 lpos[kAccBatch];
   __shared__ int lidx[kAccBatch];
   __shared__ int wcount[kAccWarps];
@@ -153,10 +165,8 @@ __global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumAr
           in = rj.x <= y && y < rj.x + M && rj.y - tx0 < sx1 && rj.y - tx0 + M > sx0;
         }
         unsigned todo = __ballot_sync(0xffffffffu, in);
-        while (todo) {
-          // The loads of up to U positions, then their sums in order.
-          vec pv[U][K], gv[U][K];
-          int cx[U], lo[U], hi[U];  // tile column of window column 0; window columns [lo, hi) of the segment
+        // The next up to U of them: issue their loads.
+        auto fetch = [&](Group& f) {
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const bool live = todo != 0;
@@ -164,42 +174,45 @@ __global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumAr
             todo &= todo - 1;
             const int ry = __shfl_sync(0xffffffffu, rj.x, src), rx = __shfl_sync(0xffffffffu, rj.y, src);
             const int i = __shfl_sync(0xffffffffu, ij, src);
-            cx[u] = rx - tx0;
-            lo[u] = max(0, sx0 - cx[u]);
-            hi[u] = live ? min(M, sx1 - cx[u]) : 0;
+            f.cx[u] = rx - tx0;
+            f.lo[u] = max(0, sx0 - f.cx[u]);
+            f.hi[u] = live ? min(M, sx1 - f.cx[u]) : 0;
             const size_t row_off = (size_t)i * MM + (size_t)(y - ry) * M;
             const float2* gp = gphi_s + row_off;
             const float2* pp = PATCH ? nullptr : s > 0 ? psi_s + row_off : a.probe + (size_t)(y - ry) * M;
-            const int x0 = (lo[u] & ~(VEC - 1)) + VEC * lane;
+            const int x0 = (f.lo[u] & ~(VEC - 1)) + VEC * lane;
 #pragma unroll
             for (int k = 0; k < K; ++k) {
               const int x = x0 + 32 * VEC * k;
-              const bool ld = x < hi[u];
-              gv[u][k] = ld ? __ldcs(reinterpret_cast<const vec*>(gp + x)) : V::zero();
+              const bool ld = x < f.hi[u];
+              f.g[u][k] = ld ? __ldcs(reinterpret_cast<const vec*>(gp + x)) : V::zero();
               if constexpr (!PATCH)
-                pv[u][k] = !ld ? V::zero()
-                               : s > 0 ? __ldcs(reinterpret_cast<const vec*>(pp + x)) : probe_load<VEC>(pp + x);
+                f.p[u][k] = !ld ? V::zero()
+                                : s > 0 ? __ldcs(reinterpret_cast<const vec*>(pp + x)) : probe_load<VEC>(pp + x);
             }
           }
+        };
+        // Add them in order.
+        auto add = [&](const Group& f) {
 #pragma unroll
           for (int u = 0; u < U; ++u) {
-            const int x0 = (lo[u] & ~(VEC - 1)) + VEC * lane;
+            const int x0 = (f.lo[u] & ~(VEC - 1)) + VEC * lane;
 #pragma unroll
             for (int e = 0; e < VEC; ++e) {
               // pixel (step k, e) is tile column cx + x0 + 32 VEC k + e (it may start at -1)
-              float2* oe = arow + (VEC == 2 ? ((cx[u] + e) & 1) * half + ((cx[u] + x0 + e) >> 1) : cx[u] + x0);
+              float2* oe = arow + (VEC == 2 ? ((f.cx[u] + e) & 1) * half + ((f.cx[u] + x0 + e) >> 1) : f.cx[u] + x0);
 #pragma unroll
               for (int k = 0; k < K; ++k) {
                 const int x = x0 + 32 * VEC * k + e;
-                if (x >= lo[u] && x < hi[u]) {
+                if (x >= f.lo[u] && x < f.hi[u]) {
                   float2* o = oe + 32 * k;
                   float2 v = *o;
-                  const float2 g = V::get(gv[u][k], e);
+                  const float2 g = V::get(f.g[u][k], e);
                   if constexpr (PATCH) {  // finished patches conj(psi) g_phi
                     v.x += g.x;
                     v.y += g.y;
                   } else {
-                    const float2 p = V::get(pv[u][k], e);
+                    const float2 p = V::get(f.p[u][k], e);
                     v.x = fmaf(p.x, g.x, fmaf(p.y, g.y, v.x));
                     v.y = fmaf(p.x, g.y, fmaf(-p.y, g.x, v.y));
                   }
@@ -208,6 +221,27 @@ __global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumAr
               }
             }
             __syncwarp();  // the next position's lanes fall on other columns
+          }
+        };
+        if constexpr (PIPE) {
+          if (!todo) continue;
+          Group f0, f1;
+          fetch(f0);
+          for (;;) {
+            const bool more1 = todo != 0;
+            if (more1) fetch(f1);
+            add(f0);
+            if (!more1) break;
+            const bool more0 = todo != 0;
+            if (more0) fetch(f0);
+            add(f1);
+            if (!more0) break;
+          }
+        } else {
+          while (todo) {
+            Group f;
+            fetch(f);
+            add(f);
           }
         }
       }
