@@ -111,7 +111,6 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
   const size_t MM = (size_t)M * M;
   size_t off = 0;
   float2* d_tw = reinterpret_cast<float2*>(base + off); off = align_up(off + M * sizeof(float2));
-  float2* d_hs = reinterpret_cast<float2*>(base + off); off = align_up(off + M * sizeof(float2));
   float2* d_h2 = reinterpret_cast<float2*>(base + off); off = align_up(off + MM * sizeof(float2));
   int* d_status = reinterpret_cast<int*>(base + off);   off = align_up(off + sizeof(int));
   double* d_loss = reinterpret_cast<double*>(base + off); off = align_up(off + sizeof(double));
@@ -131,14 +130,11 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
   float2* ws_psi = reinterpret_cast<float2*>(base + off);
 
   // Tables in FP64 on the host stack, rounded once to FP32.
-  float2 tw[128], hs[128];
+  float2 tw[128];
   const double two_pi = 6.283185307179586476925287;
   for (int k = 0; k < M; ++k) {
     const double ang = -two_pi * (double)k / (double)M;
     tw[k] = make_float2((float)std::cos(ang), (float)std::sin(ang));
-    const double f = (double)(k <= (M - 1) / 2 ? k : k - M) / ((double)M * p.pixel_A);
-    const double ph = -M_PI * p.lambda_A * p.dz_A * f * f;
-    hs[k] = make_float2((float)(std::cos(ph) / M), (float)(std::sin(ph) / M));
   }
   // The full propagator h(ky) h(kx) / M^2, staged through the stack 16 rows
   // at a time (a copy from pageable memory returns once its source is staged).
@@ -159,7 +155,6 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
   // Everything that must start at zero is cleared here: the previous call's
   // contents stay in the scratch.
   if ((e = cudaMemcpyAsync(d_tw, tw, M * sizeof(float2), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(d_hs, hs, M * sizeof(float2), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
       (e = cudaMemsetAsync(d_status, 0, sizeof(int), st)) != cudaSuccess ||
       (e = cudaMemsetAsync(d_loss, 0, sizeof(double), st)) != cudaSuccess)
     return noalloc_fail(PTYCHO_ERR_CUDA, cudaGetErrorString(e));
@@ -183,7 +178,6 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
   a.H = p.H;
   a.W = p.W;
   a.tw = d_tw;
-  a.hs = d_hs;
   a.h2 = d_h2;
   a.ws_n = chunk;
   a.ws_psi = ws_psi;
