@@ -62,8 +62,15 @@ extern "C" {
 #define PTYCHO_ERR_POSITION   -2  /* a probe window lies outside the object */
 #define PTYCHO_ERR_CUDA       -3  /* a CUDA runtime call failed */
 #define PTYCHO_ERR_NOMEM      -4  /* workspace allocation failed */
-#define PTYCHO_ERR_TIMEOUT    -5  /* a bounded device-side wait gave up (reported
-                                     by ptycho_plan_status after the stream syncs) */
+#define PTYCHO_ERR_TIMEOUT    -5  /* a bounded device-side wait gave up: between the
+                                     blocks that share a position (PTYCHO_FP32,
+                                     M = 128, few positions), or for the tensor
+                                     cores (split precisions).  The call's results
+                                     are meaningless.  Returned by the calls that
+                                     read a scalar on the host (a host loss_out,
+                                     the line search, ptycho_loss_grad_host,
+                                     ptycho_loss_grad_noalloc), else reported by
+                                     ptycho_plan_status after the stream syncs */
 #define PTYCHO_ERR_UNSUPPORTED -6 /* probe window size not supported */
 
 #define PTYCHO_FP32    0   /* all bulk complex arithmetic in FP32 */
@@ -85,14 +92,17 @@ extern "C" {
 #define PTYCHO_FLAG_TIMING      2  /* record CUDA events around every kernel
                                       family on the call's stream; read them
                                       with ptycho_plan_timing() */
-#define PTYCHO_FLAG_SELFTEST_TIMEOUT 4 /* diagnostic, split precisions only: the
-                                      kernel issues no tensor-core work and
-                                      waits for it anyway, so its bounded wait
-                                      (about 1 s) expires, it releases tensor
-                                      memory and ptycho_plan_status reports
-                                      PTYCHO_ERR_TIMEOUT.  Exercises that path
-                                      without a GPU fault; results are
-                                      meaningless. */
+#define PTYCHO_FLAG_SELFTEST_TIMEOUT 4 /* diagnostic: the split precisions' kernel
+                                      issues no tensor-core work, the PTYCHO_FP32
+                                      kernel that spreads a position over several
+                                      blocks (M = 128, few positions) no stores
+                                      between them, and both wait anyway, so the
+                                      bounded wait expires (after about 1 s; 1 ms
+                                      between blocks), tensor memory is released
+                                      and PTYCHO_ERR_TIMEOUT is reported.
+                                      Exercises that path without a GPU fault;
+                                      results are meaningless.  No effect on the
+                                      other kernels. */
 
 typedef struct {
   float re, im;
@@ -161,7 +171,7 @@ PTYCHO_API int ptycho_plan_info(ptycho_plan plan, int32_t* chunk_positions, int6
 /* Device-side status of the calls on this plan since the last read (after
  * the stream has been synchronised), and clears it: PTYCHO_OK,
  * PTYCHO_ERR_POSITION (a window outside the object was skipped),
- * PTYCHO_ERR_TIMEOUT (a bounded tensor-core wait gave up) or
+ * PTYCHO_ERR_TIMEOUT (a bounded device-side wait gave up) or
  * PTYCHO_ERR_UNSUPPORTED (a wave value left the FP16 range). */
 PTYCHO_API int ptycho_plan_status(ptycho_plan plan);
 
@@ -324,8 +334,9 @@ PTYCHO_API int ptycho_plan_timing(ptycho_plan plan, ptycho_timing* out, int32_t 
  * overlap on the GPU -- two streams, two host threads, two devices sharing
  * nothing else are fine only if they do not run at the same time on the same
  * device -- race on it.
- *   params     problem description (tile_h/tile_w as for plans; flags,
- *              workspace_bytes and ckpt_every are ignored)
+ *   params     problem description (tile_h/tile_w as for plans; flags other
+ *              than PTYCHO_FLAG_SELFTEST_TIMEOUT, workspace_bytes and
+ *              ckpt_every are ignored)
  *   pos_yx, probe, obj, meas_I, grad_obj, grad_probe: as ptycho_loss_grad,
  *              device pointers, 8-byte aligned (else PTYCHO_ERR_ARG, checked
  *              before anything is launched)
@@ -333,7 +344,7 @@ PTYCHO_API int ptycho_plan_timing(ptycho_plan plan, ptycho_timing* out, int32_t 
  * Positions are checked on the device; the call then synchronises the stream
  * and returns PTYCHO_ERR_POSITION if a window lay outside the object (that
  * window contributes nothing; the loss and gradients of the others are still
- * written).  Errors are reported by the return code only (ptycho_last_error()
+ * written), or PTYCHO_ERR_TIMEOUT if a bounded device-side wait gave up.  Errors are reported by the return code only (ptycho_last_error()
  * is not updated). */
 PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, const int32_t* pos_yx,
                                         const ptycho_c64* probe, const ptycho_c64* obj,

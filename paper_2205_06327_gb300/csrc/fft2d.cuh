@@ -187,11 +187,16 @@ struct Factors {
   uint32_t tmem;
   const float2* tw1;
   // cluster only: the mbarriers of the two row buffers, the parity of their
-  // next completion, and the device error word
+  // next completion, the device error word, and whether this warp still takes
+  // part in the exchanges
   uint64_t* mbar = nullptr;
   uint32_t phase = 0;
   int* status = nullptr;
+  int state = 0;
 };
+// Factors::state.  Muted (self-test): no exchange stores, a short wait, which
+// therefore expires.  Gave up: a wait expired.
+constexpr int kMuted = 1, kGaveUp = 2;
 constexpr int kWaitExpired = -5;  // PTYCHO_ERR_TIMEOUT
 
 template <int M>
@@ -271,6 +276,7 @@ struct ClusterCfg128 : Cfg<128> {
   // then every block has sent, so has read what the first one held.
   static constexpr uint32_t kBytes = ROWS * M * sizeof(float2);
   static constexpr long long kWaitCycles = 2000000000LL;  // about 1 s
+  static constexpr long long kShortWaitCycles = 2000000LL;  // about 1 ms
   // address of p in block `rank` of the cluster
   __device__ static __forceinline__ uint32_t peer(const void* p, int rank) {
     uint32_t r;
@@ -282,14 +288,36 @@ struct ClusterCfg128 : Cfg<128> {
                  "f"(v.x), "f"(v.y), "r"(mbar)
                  : "memory");
   }
-  // Buffer `which`'s exchange number `phase` has arrived.
+  // Buffer `which`'s exchange number `phase` has arrived.  A warp whose wait
+  // expires reports it and gives up: it neither waits nor arms an mbarrier nor
+  // stores into another block from then on (what it computes is meaningless), so
+  // the other blocks' next wait expires too and the kernel ends within two
+  // limits.  An mbarrier is only armed again by a thread that saw its last phase
+  // complete.
   __device__ static __forceinline__ void arrived(Factors& f, int which) {
+    if (f.state & kGaveUp) return;
     uint64_t* mbar = f.mbar + which;
     if (threadIdx.x == 0)
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(mbar)), "r"(kBytes)
                    : "memory");
-    if (!tc::mbar_wait_bounded(mbar, f.phase >> which & 1u, kWaitCycles)) *f.status = kWaitExpired;
+    const long long limit = f.state & kMuted ? kShortWaitCycles : kWaitCycles;
+    const bool done = tc::mbar_wait_bounded(mbar, f.phase >> which & 1u, limit);
+    if (!__all_sync(0xffffffffu, done)) {
+      *f.status = kWaitExpired;
+      f.state |= kGaveUp;
+      return;
+    }
     f.phase ^= 1u << which;
+  }
+  // Before a block gives its memory back: no block leaves while another may
+  // still store into it.  A block whose exchanges all arrived has nothing in
+  // flight towards it; one that gave up lets late stores of the exchange it left
+  // land first (its peers have issued theirs by the barrier).
+  __device__ static __forceinline__ void leave(const Factors& f) {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    if (f.state & kGaveUp)
+      for (int which = 0; which < 2; ++which)
+        tc::mbar_wait_bounded(f.mbar + which, f.phase >> which & 1u, kShortWaitCycles);
   }
   __device__ static __forceinline__ void put_loss(double* red, int w, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(peer(red + w, 0)), "d"(v) : "memory");
@@ -368,6 +396,9 @@ __device__ __forceinline__ int opaque(int x) {
 template <class C, int J, bool FAR>
 __device__ __forceinline__ void xch_store(const float2 (&v)[C::V], float2* sm, const Factors& f, int t) {
   using P = PassShape<C, J>;
+  if constexpr (C::CL > 1 && FAR) {
+    if (f.state) return;  // muted, or gave up
+  }
   t = opaque(t);
   static_for<0, P::Q>([&](auto qq) {
     constexpr int q = decltype(qq)::value;

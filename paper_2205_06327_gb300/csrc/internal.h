@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "../../include/ptycho.h"
+
 namespace ptycho {
 
 // Programmatic dependent launch: a kernel launched with launch_after may start
@@ -15,6 +17,13 @@ namespace ptycho {
 // constant tables, so completion carries over from kernel to kernel.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// What a non-zero device error word stands for.
+inline const char* status_text(int h) {
+  if (h == PTYCHO_ERR_TIMEOUT) return "a bounded device-side wait gave up";
+  if (h == PTYCHO_ERR_UNSUPPORTED) return "a wave value left the FP16 range (|x| >= 60000)";
+  return "a probe window outside the object was skipped on the device";
+}
 
 template <class... P, class... A>
 cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
@@ -71,7 +80,8 @@ struct ChainArgs {
   int* status;            // device error word
   int* pos_status;        // where a window outside the object is flagged (PTYCHO_ERR_POSITION):
                           // the error word, or a word nobody reads when the host checks
-  int selftest_timeout;   // PTYCHO_FLAG_SELFTEST_TIMEOUT: the split-product kernel issues no MMAs
+  int selftest_timeout;   // PTYCHO_FLAG_SELFTEST_TIMEOUT: the split-product kernel issues no MMAs, the
+                          // cluster chain no exchange stores
 };
 
 // Gradient-mode chains of several problems (same window M = 64 or 128, FP32,

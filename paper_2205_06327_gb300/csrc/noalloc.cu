@@ -186,6 +186,7 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
   a.loss_part = loss_part;
   a.status = d_status;
   a.pos_status = d_status;
+  a.selftest_timeout = (p.flags & PTYCHO_FLAG_SELFTEST_TIMEOUT) ? 1 : 0;
   const bool want_grad = grad_obj || grad_probe;
   for (int c0 = 0, ci = 0; c0 < p.N; c0 += chunk, ++ci) {
     const int n = p.N - c0 < chunk ? p.N - c0 : chunk;
@@ -224,6 +225,6 @@ extern "C" PTYCHO_API int ptycho_loss_grad_noalloc(const ptycho_params* params, 
       (e = cudaMemcpyAsync(loss_out, d_loss, sizeof(double), cudaMemcpyDefault, st)) != cudaSuccess ||
       (e = cudaStreamSynchronize(st)) != cudaSuccess)
     return noalloc_fail(PTYCHO_ERR_CUDA, cudaGetErrorString(e));
-  if (status) return noalloc_fail(PTYCHO_ERR_POSITION, "a probe window lies outside the object");
+  if (status) return noalloc_fail(status, status_text(status));
   return PTYCHO_OK;
 }

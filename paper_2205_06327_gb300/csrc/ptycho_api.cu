@@ -165,6 +165,7 @@ constexpr int64_t kDefaultWorkspace = 8ll << 30;
 constexpr int64_t kGmWaveBytes = 64ll << 20;
 constexpr int kProbeSplit = 32;
 constexpr int kNormParts = 512;
+constexpr int kStatusSlot = 4;  // the scalar slot that holds the device error words
 
 }  // namespace
 
@@ -185,13 +186,13 @@ struct ptycho_plan_s {
   float2* gp_part = nullptr;  // [kProbeSplit][M][M]
   double* loss_part = nullptr;  // [chunk][loss_parts]
   int loss_parts = 1;           // loss parts per position (generic-window path: its line blocks)
-  double* d_scal = nullptr;   // [8]: 0 loss, 1 |gO|^2, 2 |gP|^2, 3 trial loss
+  double* d_scal = nullptr;   // [8]: 0 loss, 1 |gO|^2, 2 |gP|^2, 3 trial loss, 4 the words of d_status
   double* norm_part = nullptr;  // [kNormParts]
-  int* d_status = nullptr;    // [2]: the error word, and the word of host-checked plans' chains
+  int* d_status = nullptr;    // [2]: the error word, and the word of host-checked plans' chains; kept
+                              // behind the scalars, so that one copy brings both (read_scalars)
   cudaEvent_t ev_check = nullptr;  // the positions have reached h_pos
   int* h_pos = nullptr;       // pinned, [N][2]
   double* h_scal = nullptr;   // pinned, [8]
-  int* h_flag = nullptr;      // pinned, [1]: the device error word, read by the synchronous calls
   // gradient-descent step buffers (allocated on first use)
   float2* g_obj = nullptr;
   float2* g_probe = nullptr;
@@ -241,7 +242,6 @@ void free_plan(ptycho_plan pl) {
   cudaFree(pl->loss_part);
   cudaFree(pl->d_scal);
   cudaFree(pl->norm_part);
-  cudaFree(pl->d_status);
   cudaFree(pl->g_obj);
   cudaFree(pl->g_probe);
   cudaFree(pl->d_cplanes);
@@ -260,7 +260,6 @@ void free_plan(ptycho_plan pl) {
   if (pl->copy) cudaStreamDestroy(pl->copy);
   if (pl->h_pos) cudaFreeHost(pl->h_pos);
   if (pl->h_scal) cudaFreeHost(pl->h_scal);
-  if (pl->h_flag) cudaFreeHost(pl->h_flag);
   delete pl;
 }
 
@@ -308,11 +307,7 @@ int validate_params(const ptycho_params& p) {
 int check_windows(const ptycho_params& p, const int32_t* h_pos);
 
 // The error a non-zero device error word stands for.
-int status_fail(int h) {
-  if (h == PTYCHO_ERR_TIMEOUT) return fail(h, "a bounded tensor-core wait gave up on the device");
-  if (h == PTYCHO_ERR_UNSUPPORTED) return fail(h, "a wave value left the FP16 range (|x| >= 60000)");
-  return fail(h, "a probe window outside the object was skipped on the device");
-}
+int status_fail(int h) { return fail(h, status_text(h)); }
 
 // Positions check on the host (pinned copy) unless the plan asks for the
 // asynchronous device-side check only.  It comes in two halves so that the
@@ -618,13 +613,24 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
   return PTYCHO_OK;
 }
 
+// The scalars in h_scal, once st is done.  A wait that gave up leaves every
+// number of the call meaningless: a call that reads scalars reports it (the
+// other device errors concern single positions or values and wait for
+// ptycho_plan_status, which reports this one as well).
+int read_scalars(ptycho_plan pl, cudaStream_t st) {
+  CUDA_TRY(cudaMemcpyAsync(pl->h_scal, pl->d_scal, (kStatusSlot + 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
+  int h;
+  std::memcpy(&h, pl->h_scal + kStatusSlot, sizeof h);
+  return h == PTYCHO_ERR_TIMEOUT ? status_fail(h) : PTYCHO_OK;
+}
+
 int deliver_loss(ptycho_plan pl, int slot, double* loss_out, cudaStream_t st) {
   if (!loss_out) return PTYCHO_OK;
   if (is_device_ptr(loss_out)) {
     CUDA_TRY(cudaMemcpyAsync(loss_out, pl->d_scal + slot, sizeof(double), cudaMemcpyDeviceToDevice, st));
   } else {
-    CUDA_TRY(cudaMemcpyAsync(pl->h_scal + slot, pl->d_scal + slot, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
+    if (const int rc = read_scalars(pl, st)) return rc;
     *loss_out = pl->h_scal[slot];
   }
   return PTYCHO_OK;
@@ -754,7 +760,7 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
   if (!rc) rc = dev_alloc(&pl->loss_part, (size_t)pl->chunk * pl->loss_parts, "loss partials");
   if (!rc) rc = dev_alloc(&pl->d_scal, 8, "scalars");
   if (!rc) rc = dev_alloc(&pl->norm_part, kNormParts, "norm partials");
-  if (!rc) rc = dev_alloc(&pl->d_status, 2, "status");
+  if (!rc) pl->d_status = reinterpret_cast<int*>(pl->d_scal + kStatusSlot);
   std::vector<uint32_t> planes;
   if (!rc && p.precision != PTYCHO_FP32) {
     planes = build_tc_planes(p, p.precision == PTYCHO_FP16X3);
@@ -778,8 +784,7 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
     return cuda_fail(e, "plane upload");
   }
   if (cudaMallocHost(&pl->h_pos, sizeof(int32_t) * 2 * (size_t)n) != cudaSuccess ||
-      cudaMallocHost(&pl->h_scal, sizeof(double) * 8) != cudaSuccess ||
-      cudaMallocHost(&pl->h_flag, sizeof(int)) != cudaSuccess) {
+      cudaMallocHost(&pl->h_scal, sizeof(double) * 8) != cudaSuccess) {
     cudaGetLastError();
     free_plan(pl);
     return fail(PTYCHO_ERR_NOMEM, "pinned host allocation failed");
@@ -789,7 +794,6 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
       (e = cudaMemcpy(pl->d_hs, hs.data(), M * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (!h2.empty() &&
        (e = cudaMemcpy(pl->d_h2, h2.data(), h2.size() * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (e = cudaMemset(pl->d_status, 0, 2 * sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(pl->d_scal, 0, 8 * sizeof(double))) != cudaSuccess) {
     free_plan(pl);
     return cuda_fail(e, "table upload");
@@ -924,8 +928,7 @@ int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho
   if (line_search) {
     TIMED(K_OTHER, 2, launch_norm2(plan->g_obj, nO, plan->norm_part, kNormParts, plan->d_scal, 1, st));
     TIMED(K_OTHER, 2, launch_norm2(plan->g_probe, nP, plan->norm_part, kNormParts, plan->d_scal, 2, st));
-    CUDA_TRY(cudaMemcpyAsync(plan->h_scal, plan->d_scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
+    if ((rc = read_scalars(plan, st))) return rc;
     const double F0 = plan->h_scal[0];
     const double dec = alpha_obj * plan->h_scal[1] + alpha_probe * plan->h_scal[2];
     bool accepted = false;
@@ -933,8 +936,7 @@ int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho
       rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, nullptr, nullptr, 3, plan->g_obj,
                          (float)(-t * alpha_obj), plan->g_probe, (float)(-t * alpha_probe), st);
       if (rc) return rc;
-      CUDA_TRY(cudaMemcpyAsync(plan->h_scal + 3, plan->d_scal + 3, sizeof(double), cudaMemcpyDeviceToHost, st));
-      CUDA_TRY(cudaStreamSynchronize(st));
+      if ((rc = read_scalars(plan, st))) return rc;
       if (plan->h_scal[3] <= F0 - 1e-4 * t * dec) {
         accepted = true;
         break;
@@ -1174,10 +1176,13 @@ int loss_grad_host_impl(ptycho_plan plan, const int32_t* pos_yx, const ptycho_c6
   }
   if (grad_obj) CUDA_TRY(cudaMemcpyAsync(grad_obj, pl->x_gO, sizeof(float2) * nO, cudaMemcpyDeviceToHost, st));
   if (grad_probe) CUDA_TRY(cudaMemcpyAsync(grad_probe, pl->x_gP, sizeof(float2) * MM, cudaMemcpyDeviceToHost, st));
-  // The call is synchronous, so it reports the device error word itself.
-  CUDA_TRY(cudaMemcpyAsync(pl->h_flag, pl->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
-  if ((rc = deliver_loss(pl, 0, loss_out, st))) return rc;  // synchronises st
-  if (const int h = *pl->h_flag) {
+  // The call is synchronous, so it reports the device error word itself (and clears it).
+  rc = read_scalars(pl, st);
+  if (rc && rc != PTYCHO_ERR_TIMEOUT) return rc;
+  *loss_out = pl->h_scal[0];
+  int h;
+  std::memcpy(&h, pl->h_scal + kStatusSlot, sizeof h);
+  if (h) {
     CUDA_TRY(cudaMemsetAsync(pl->d_status, 0, sizeof(int), st));
     CUDA_TRY(cudaStreamSynchronize(st));
     return status_fail(h);

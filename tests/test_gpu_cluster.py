@@ -84,3 +84,55 @@ def test_cluster_recompute_and_window_outside(dev, S, L):
     assert abs(l.item() - F) <= TOL_FP32 * F
     assert rel_l2(go.cpu().numpy(), gO) <= TOL_FP32 and rel_l2(gp.cpu().numpy(), gP) <= TOL_FP32
     plan.close()
+
+
+@pytest.mark.parametrize("n,S,L", [(1, 1, 0), (3, 4, 0), (2, 5, 2)])
+def test_cluster_wait_that_expires_is_reported(dev, n, S, L):
+    """With PTYCHO_FLAG_SELFTEST_TIMEOUT the blocks of a cluster send nothing
+    and wait for one another anyway: the short wait expires, the kernel ends (no
+    further waits, however many exchanges follow), an asynchronous call leaves
+    PTYCHO_ERR_TIMEOUT for ptycho_plan_status, calls that read a scalar on the
+    host return it, a line search leaves the unknowns alone, and the next
+    evaluation on the GPU is right."""
+    import ctypes as C
+
+    from paper_2205_06327_gb300 import _lib
+    wl = synth.workload_random(128, S, 1, n, 9, seed=830 + S, amp_jitter=0.1)
+    I = (measurements(wl) * 1.1).astype(np.float32)
+    wl.obj = start_object(wl, "perturbed", S)
+    pos, probe, obj, meas = _tensors(wl, I, dev)
+    lib = _lib.load()
+    p = _lib.PtychoParams(M=wl.M, S=wl.S, H=wl.H, W=wl.W, N=wl.N, lambda_A=wl.lambda_A, dz_A=wl.dz_A,
+                          pixel_A=wl.pixel_A, ckpt_every=L, flags=_lib.PTYCHO_FLAG_SELFTEST_TIMEOUT)
+    h = C.c_void_p()
+    st = torch.cuda.current_stream(dev).cuda_stream
+    assert lib.ptycho_plan_create(C.byref(h), C.byref(p)) == _lib.PTYCHO_OK
+    gO, gP = torch.empty_like(obj), torch.empty_like(probe)
+    loss = torch.zeros((), dtype=torch.float64, device=dev)
+    args = (pos.data_ptr(), probe.data_ptr(), obj.data_ptr(), meas.data_ptr())
+    assert lib.ptycho_loss_grad(h, *args, loss.data_ptr(), gO.data_ptr(), gP.data_ptr(), st) == _lib.PTYCHO_OK
+    torch.cuda.synchronize()
+    assert lib.ptycho_plan_status(h) == _lib.PTYCHO_ERR_TIMEOUT
+    assert lib.ptycho_plan_status(h) == _lib.PTYCHO_OK  # reading clears it
+    hl, t = C.c_double(0.0), C.c_double(0.0)
+    for grads in ((gO.data_ptr(), gP.data_ptr()), (None, None)):
+        assert lib.ptycho_loss_grad(h, *args, C.addressof(hl), *grads, st) == _lib.PTYCHO_ERR_TIMEOUT
+        assert b"gave up" in lib.ptycho_last_error()
+        assert lib.ptycho_plan_status(h) == _lib.PTYCHO_ERR_TIMEOUT
+    probe2, obj2 = probe.clone(), obj.clone()
+    assert lib.ptycho_step(h, pos.data_ptr(), probe2.data_ptr(), obj2.data_ptr(), meas.data_ptr(), 0.1, 0.1, 1,
+                           None, C.addressof(t), st) == _lib.PTYCHO_ERR_TIMEOUT
+    torch.cuda.synchronize()
+    assert torch.equal(probe2, probe) and torch.equal(obj2, obj)
+    assert lib.ptycho_plan_destroy(h) == _lib.PTYCHO_OK
+    if L == 0:
+        assert lib.ptycho_loss_grad_noalloc(C.byref(p), *args, C.addressof(hl), gO.data_ptr(), gP.data_ptr(),
+                                            st) == _lib.PTYCHO_ERR_TIMEOUT
+    p.flags = 0
+    assert lib.ptycho_plan_create(C.byref(h), C.byref(p)) == _lib.PTYCHO_OK
+    assert lib.ptycho_loss_grad(h, *args, C.addressof(hl), gO.data_ptr(), gP.data_ptr(), st) == _lib.PTYCHO_OK
+    assert lib.ptycho_plan_status(h) == _lib.PTYCHO_OK
+    F, rO, rP = orc.loss_grad(c64(wl.probe), c64(wl.obj), wl.pos, I.astype(np.float64), propagator(wl))
+    assert abs(hl.value - F) <= TOL_FP32 * F
+    assert rel_l2(gO.cpu().numpy(), rO) <= TOL_FP32 and rel_l2(gP.cpu().numpy(), rP) <= TOL_FP32
+    assert lib.ptycho_plan_destroy(h) == _lib.PTYCHO_OK
