@@ -19,6 +19,7 @@
 #pragma once
 
 #include "../../include/ptycho.h"
+#include "bounds.h"
 #include "fft2d.cuh"
 #include "internal.h"
 
@@ -201,8 +202,8 @@ struct GmBlock {
   bool cols;
 
   __device__ __forceinline__ int at(int li, int i) const { return cols ? i * M + (l0 + li) : (l0 + li) * M + i; }
-  __device__ __forceinline__ int obj_at(int li, int i) const {
-    return cols ? i * a.W + (l0 + li) : (l0 + li) * a.W + i;
+  __device__ __forceinline__ int64_t obj_at(int li, int i) const {
+    return cols ? window_at(i, l0 + li, a.W) : window_at(l0 + li, i, a.W);
   }
   __device__ __forceinline__ const float2* obj_window(const float2* o) const {
     return o + (size_t)g.s * a.H * a.W + (size_t)r.x * a.W + r.y;
@@ -213,10 +214,11 @@ struct GmBlock {
   // the call has one), the adjoint keeps g_phi_s and multiplies by conj(O_s).
   template <int KIND, int R>
   __device__ __forceinline__ void transmit(float2 (&x)[R], int li, int i0, int di) const {
-    const float2* ow = obj_window(a.obj);
+    const int64_t step = cols ? window_at(di, 0, a.W) : di;  // from one of the elements to the next
+    const float2* ow = obj_window(a.obj) + obj_at(li, i0);
     float2 o[R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) o[q] = __ldg(ow + obj_at(li, i0 + q * di));
+    for (int q = 0; q < R; ++q, ow += step) o[q] = __ldg(ow);
     if constexpr (KIND == GM_FWD) {
       if (g.from_probe && a.probe_dir) {
 #pragma unroll
@@ -227,10 +229,10 @@ struct GmBlock {
         }
       }
       if (a.obj_dir) {
-        const float2* dw = obj_window(a.obj_dir);
+        const float2* dw = obj_window(a.obj_dir) + obj_at(li, i0);
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-          const float2 d = __ldg(dw + obj_at(li, i0 + q * di));
+        for (int q = 0; q < R; ++q, dw += step) {
+          const float2 d = __ldg(dw);
           o[q].x = fmaf(a.obj_step, d.x, o[q].x);
           o[q].y = fmaf(a.obj_step, d.y, o[q].y);
         }

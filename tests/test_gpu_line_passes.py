@@ -61,3 +61,24 @@ def test_line_pass_window_outside_contributes_nothing(dev, M):
     with pytest.raises(PtychoError):
         plan.status()
     assert abs(l - F) <= TOL_FP32 * F and rel_l2(go, gO) <= TOL_FP32 and rel_l2(gp, gP) <= TOL_FP32
+
+
+@pytest.mark.parametrize("M,W", [(1024, 2100000), (1152, 1880000)])  # an instance, the runtime radix schedule
+def test_line_pass_window_of_a_very_wide_object(dev, M, W):
+    """A window of an object so wide that its last rows lie 2^31 pixels and more
+    from its first: the same window alone gives the same result bit for bit."""
+    from paper_2205_06327_gb300 import api
+    g = torch.Generator(device=dev).manual_seed(M)
+    win = torch.exp(0.3j * torch.rand(1, M, M, device=dev, generator=g))
+    meas = torch.rand(1, M, M, device=dev, generator=g) / M
+    probe = to_dev(synth.defocused_probe(M, 0.15, np.pi * 0.15 * M, 1.0, energy=float(M)), torch.complex64, dev)
+    wide = torch.ones(1, M, W, dtype=torch.complex64, device=dev)
+    wide[:, :, W - M:] = win
+    out = []
+    for obj, x, width in ((win, 0, M), (wide, W - M, W)):
+        plan = api.Plan(api.Geometry(M, 1, M, width, 1), dev)
+        loss, gO, gP = plan.loss_grad(torch.tensor([[0, x]], dtype=torch.int32, device=dev), probe, obj, meas)
+        out.append((loss, gO[:, :, x:x + M].clone(), gP))
+        assert x == 0 or not torch.count_nonzero(gO[:, :, :x])
+        plan.close()
+    assert all(torch.equal(a, b) for a, b in zip(*out))
