@@ -27,6 +27,7 @@
 // the parked state and parks the state again (segment 0: the probe gradient).
 // The host accumulates each segment's patches into the object gradient
 // before the next launch overwrites them.
+#include "bounds.h"
 #include "fft2d.cuh"
 #include "internal.h"
 #include "../../include/ptycho.h"
@@ -141,11 +142,20 @@ int chain_threads(int M) { return M == 128 ? Cfg<128>::T : Cfg<64>::T; }
 
 // The exchange buffer, the pass-1 twiddle table, the loss partials of the
 // position's warps and the tensor-memory address.
+//
+// A cluster's block holds tensor memory while it waits for the other blocks of
+// its cluster, and the allocation waits without limit.  If more of them were
+// resident on an SM than its tensor memory serves, two clusters could each hold
+// columns that the other one's blocks wait for, for ever.  Registers (218 to
+// 241 a thread) happen to allow four blocks; shared memory makes it certain,
+// also for launches of several streams together.
 template <class C>
 static constexpr size_t chain_smem() {
-  return (C::kSmemWave + 16 * (size_t)tw1_stride<C>()) * sizeof(float2) + (C::T / 32 + 1) * sizeof(double) +
-         (C::CL > 1 ? 2 * sizeof(uint64_t) : 0);
+  const size_t need = (C::kSmemWave + 16 * (size_t)tw1_stride<C>()) * sizeof(float2) +
+                      (C::T / 32 + 1) * sizeof(double) + (C::CL > 1 ? 2 * sizeof(uint64_t) : 0);
+  return C::CL > 1 ? smem_for_at_most(kTmemColumns / kTmemTake<C>, need) : need;
 }
+static_assert(chain_smem<ClusterCfg128>() <= 48 << 10, "a launch may ask for it without raising the kernel's limit");
 
 size_t chain_smem_bytes(int M) { return M == 128 ? chain_smem<Cfg<128>>() : chain_smem<Cfg<64>>(); }
 

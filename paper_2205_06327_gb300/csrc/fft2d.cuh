@@ -356,6 +356,10 @@ struct Cfg<64> {
   }
 };
 
+// Tensor-memory columns a block takes: 128 per 4 warps.
+template <class C>
+constexpr int kTmemTake = C::TB < 128 ? 128 : C::TB;
+
 // The same with half the factors fetched at a time.  Fewer, wider fetches wait
 // less but hold more registers: 576 positions, M = 128, 16 slices, gradient
 // 1606 us with 8 at a time, 1587 with 16 (4560 positions in recompute mode 27.3

@@ -27,3 +27,16 @@ def test_window_offsets_of_wide_objects(tmp_path, M, W):
     at = _run(tmp_path, f'std::printf("%lld %lld\\n", (long long)window_at({M - 1}, {M - 1}, {W}), '
                         f'(long long)window_at({M - 1}, 0, {W}));')
     assert at == [(M - 1) * W + M - 1, (M - 1) * W]
+
+
+@pytest.mark.parametrize("blocks", [1, 2, 4, 8])
+@pytest.mark.parametrize("need", [1000, 38000, 60000])
+def test_shared_memory_limits_the_resident_blocks(tmp_path, blocks, need):
+    """One block more than the limit does not fit on an SM; the limit itself fits
+    unless the kernel's own need is larger.  The cluster chain's limit is what
+    tensor memory serves."""
+    smem, cols, sm, block = _run(tmp_path, f'std::printf("%zu %d %zu %zu\\n", smem_for_at_most({blocks}, {need}), '
+                                           'kTmemColumns, kSmShared, kBlockShared);')
+    assert smem >= need and smem % 128 in (0, need % 128) and (blocks + 1) * (smem + block) > sm
+    assert smem == need or blocks * (smem + block) <= sm
+    assert cols // 128 == 4
