@@ -41,6 +41,10 @@
  *
  * Errors: every entry point returns PTYCHO_OK (0) or a negative code and
  * records a message retrievable with ptycho_last_error() (per host thread).
+ * Without PTYCHO_FLAG_ASYNC_CHECK the positions are checked on the host while
+ * the first kernels run.  A call refused for a window outside the object
+ * (PTYCHO_ERR_POSITION) writes none of the caller's arrays and returns once
+ * those kernels are done, so its inputs may be freed or rewritten at once.
  */
 #ifndef PTYCHO_H_
 #define PTYCHO_H_

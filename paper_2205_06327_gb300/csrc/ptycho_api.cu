@@ -336,6 +336,13 @@ int check_positions(ptycho_plan pl, const int32_t* pos, cudaStream_t st) {
   return rc ? rc : end_check(pl);
 }
 
+// A host-checked call that fails after begin_check returns once what it has
+// enqueued is done: the caller may free or rewrite its arrays at once.
+int settled(ptycho_plan pl, int rc, cudaStream_t st) {
+  if (rc && !(pl->p.flags & PTYCHO_FLAG_ASYNC_CHECK)) cudaStreamSynchronize(st);
+  return rc;
+}
+
 // Every window inside the object: 0 <= y <= H - M, 0 <= x <= W - M.
 int check_windows(const ptycho_params& p, const int32_t* h_pos) {
   for (int i = 0; i < p.N; ++i) {
@@ -900,7 +907,7 @@ int loss_grad_impl(ptycho_plan plan, const int32_t* pos_yx, const ptycho_c64* pr
   if ((rc = begin_check(plan, pos_yx, st))) return rc;
   rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, reinterpret_cast<float2*>(grad_obj),
                      reinterpret_cast<float2*>(grad_probe), 0, nullptr, 0.f, nullptr, 0.f, st, 0, nullptr, true);
-  if (rc) return rc;
+  if (rc) return settled(plan, rc, st);
   return deliver_loss(plan, 0, loss_out, st);
 }
 
@@ -917,11 +924,11 @@ int step_impl(ptycho_plan plan, const int32_t* pos_yx, ptycho_c64* probe, ptycho
     return rc;
   if ((rc = begin_check(plan, pos_yx, st))) return rc;
   const size_t nO = (size_t)p.S * p.H * p.W, nP = (size_t)p.M * p.M;
-  if (!plan->g_obj && (rc = dev_alloc(&plan->g_obj, nO, "step object gradient"))) return rc;
-  if (!plan->g_probe && (rc = dev_alloc(&plan->g_probe, nP, "step probe gradient"))) return rc;
-  rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, plan->g_obj, plan->g_probe, 0, nullptr, 0.f, nullptr, 0.f, st,
-                     0, nullptr, true);
-  if (rc) return rc;
+  if ((!plan->g_obj && (rc = dev_alloc(&plan->g_obj, nO, "step object gradient"))) ||
+      (!plan->g_probe && (rc = dev_alloc(&plan->g_probe, nP, "step probe gradient"))) ||
+      (rc = run_loss_grad(plan, pos_yx, probe, obj, meas_I, plan->g_obj, plan->g_probe, 0, nullptr, 0.f, nullptr, 0.f,
+                          st, 0, nullptr, true)))
+    return settled(plan, rc, st);
   if ((rc = deliver_loss(plan, 0, loss_out, st))) return rc;
   ptycho_plan pl = plan;
   double t = 1.0;
