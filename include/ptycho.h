@@ -265,11 +265,12 @@ PTYCHO_API int ptycho_step_accumulate(ptycho_plan plan, const int32_t* pos_yx, p
  * problems' work is enqueued on `stream` (part of it on a stream of the
  * library's, forked from `stream` and joined back to it), so one call can be
  * captured in one CUDA graph when every plan uses PTYCHO_FLAG_ASYNC_CHECK: the
- * problems the register-resident kernels do not take run in order; beside
- * them, the FP32 problems with M = 64 or 128 that keep every wave, grouped by
+ * problems the register-resident kernels do not take run first, in order,
+ * then the FP32 problems with M = 64 or 128 that keep every wave, grouped by
  * window, whose chains of chunk r run in one launch per group (up to 16
  * problems per launch), each followed by that problem's reductions of the
- * chunk.  So no problem may read what another one writes.  The
+ * chunk.  Where no problem of one kind writes memory that one of the other
+ * kind uses, the two kinds run side by side.  The
  * call never synchronises (unless a plan lacks PTYCHO_FLAG_ASYNC_CHECK):
  * loss_out must be a device pointer or NULL.  Results are bit-identical to
  * the single-problem calls.  On an error the message names the problem; the

@@ -1070,17 +1070,54 @@ int run_multi_fused(const ptycho_problem* probs, const std::vector<int>& idx, bo
   return PTYCHO_OK;
 }
 
+// Does a problem in `fused` write memory that another problem of the call reads
+// or writes, or read what one writes?
+bool fused_share(const ptycho_problem* probs, int32_t n, const std::vector<int>& fused, bool step) {
+  struct Range {
+    uintptr_t begin, end;
+  };
+  std::vector<Range> written[2], touched[2];  // by the others, by the fused
+  for (int32_t i = 0, k = 0; i < n; ++i) {
+    const bool f = k < (int32_t)fused.size() && fused[k] == i;
+    k += f;
+    const ptycho_problem& q = probs[i];
+    const ptycho_params& p = q.plan->p;
+    const size_t MM = (size_t)p.M * p.M, nO = (size_t)p.S * p.H * p.W;
+    auto add = [&](const void* ptr, size_t bytes, bool write) {
+      if (!ptr || !bytes) return;
+      const uintptr_t b = reinterpret_cast<uintptr_t>(ptr);
+      touched[f].push_back({b, b + bytes});
+      if (write) written[f].push_back({b, b + bytes});
+    };
+    add(q.pos_yx, 2 * sizeof(int32_t) * (size_t)p.N, false);
+    add(q.meas_I, sizeof(float) * MM * (size_t)p.N, false);
+    add(q.probe, sizeof(float2) * MM, step);
+    add(q.obj, sizeof(float2) * nO, step);
+    add(q.loss_out, sizeof(double), true);
+    if (!step) {
+      add(q.grad_obj, sizeof(float2) * nO, true);
+      add(q.grad_probe, sizeof(float2) * MM, true);
+    }
+  }
+  for (int f = 0; f < 2; ++f)
+    for (const Range& w : written[f])
+      for (const Range& r : touched[1 - f])
+        if (w.begin < r.end && r.begin < w.end) return true;
+  return false;
+}
+
 // The problems of one call: those in `fused` through run_multi_fused, the
-// others through fn(problem), in order, on st.  With both kinds present the
-// fused ones run on a side stream forked from st and joined back: their chains
-// keep their waves on chip, so they fill the SMs that the line passes' partial
-// waves leave idle without competing for the L2 (one problem per window class,
-// 1428 positions, graph replay: 3171 -> 3049 us).  Each kind by itself stays on one
-// stream: the line passes size their chunks to the L2.
+// others through fn(problem), in order, before them.  With both kinds present
+// the fused ones run on a side stream forked from st and joined back: their
+// chains keep their waves on chip, so they fill the SMs that the line passes'
+// partial waves leave idle without competing for the L2 (one problem per window
+// class, 1428 positions, graph replay: 3171 -> 3049 us).  Each kind by itself
+// stays on one stream: the line passes size their chunks to the L2.  Problems
+// that share memory that one of them writes keep the order on st.
 template <class F>
 int run_multi(const ptycho_problem* probs, int32_t n, const std::vector<int>& fused, bool step, double a_o, double a_p,
               cudaStream_t st, F&& fn) {
-  const bool fork = !fused.empty() && (int32_t)fused.size() < n;
+  const bool fork = !fused.empty() && (int32_t)fused.size() < n && !fused_share(probs, n, fused, step);
   ptycho_plan fp = fork ? probs[fused[0]].plan : nullptr;
   cudaStream_t fst = st;
   if (fork) {
@@ -1088,7 +1125,7 @@ int run_multi(const ptycho_problem* probs, int32_t n, const std::vector<int>& fu
     CUDA_TRY(cudaEventRecord(fp->ev_fork, st));
     CUDA_TRY(cudaStreamWaitEvent(fst, fp->ev_fork, 0));
   }
-  int rc = run_multi_fused(probs, fused, step, a_o, a_p, fst);
+  int rc = fork ? run_multi_fused(probs, fused, step, a_o, a_p, fst) : PTYCHO_OK;
   for (int32_t i = 0, k = 0; !rc && i < n; ++i) {
     if (k < (int32_t)fused.size() && fused[k] == i) {
       ++k;
@@ -1100,7 +1137,7 @@ int run_multi(const ptycho_problem* probs, int32_t n, const std::vector<int>& fu
     CUDA_TRY(cudaEventRecord(fp->ev_join, fst));
     CUDA_TRY(cudaStreamWaitEvent(st, fp->ev_join, 0));
   }
-  return rc;
+  return rc || fork ? rc : run_multi_fused(probs, fused, step, a_o, a_p, st);
 }
 
 // ptycho_loss_grad_host: host arrays in and out.  The inputs are staged in
