@@ -209,16 +209,32 @@ static cudaError_t launch_cluster(ChainMode mode, const ChainArgs& a, cudaStream
   }
 }
 
-// One launch of at most kClusterMax positions takes the cluster kernel (results
-// are the same bit for bit).  us of a gradient chain of 16 slices, one block
-// against one cluster per position: 1 position 311 -> 168, 10 311 -> 174, 19
-// 312 -> 205, 38 312 -> 255; with two blocks per SM and more the blocks of
-// different positions compete (76 positions 312 -> 520).
-constexpr int kClusterMax = 48;
+// Does a launch take the cluster kernel?  Results are the same bit for bit, so
+// this is where it is the faster one.  us of an evaluation, one block / one
+// cluster per position: 16 slices, 1 position 332 / 198, 24 352 / 248, 40 358 /
+// 297, 48 362 / 332 (76: the chain alone 312 / 520, as the blocks of different
+// positions compete); 48 positions of 4 slices 128 / 123, of 3 109 / 109; forward
+// model of 16 slices, 48 positions 137 / 134.  Gradients of one or two slices
+// have few exchanges to win by: 2 slices, 16 positions 77 / 74, 32 91 / 92, 48 90
+// / 94; one slice, 48 positions 65 / 68.
+// As a chunk's tail it takes SMs from the accumulation of the chunk's `beside`
+// full waves, which runs at the same time, the more the longer that lasts: 16
+// slices, 152 + 48 positions 693 / 660, 304 + 32 1022 / 982, 304 + 48 1029 /
+// 1063, 456 + 16 1386 / 1348, 456 + 48 1362 / 1477, 608 + 16 1708 / 1740; 8
+// slices, 152 + 32 380 / 360, 152 + 48 385 / 401; 4 slices, 152 + 16 219 / 209,
+// 304 + 16 317 / 323; 2 slices, 152 + 8 142 / 148.
+bool cluster_faster(ChainMode mode, const ChainArgs& a, int beside) {
+  int most = 48;
+  if (beside > 0)
+    most = a.S < 4 ? 0 : (a.S < 12 ? 4 * a.S : 48) - 16 * (beside - 1);
+  else if (mode != MODE_FORWARD && mode != MODE_LOSS && a.S < 3)
+    most = a.S == 2 ? 16 : 0;
+  return a.n_pos <= most;
+}
 
-cudaError_t launch_chain(int M, ChainMode mode, const ChainArgs& a, cudaStream_t st) {
+cudaError_t launch_chain(int M, ChainMode mode, const ChainArgs& a, cudaStream_t st, int beside) {
   if (a.n_pos <= 0) return cudaSuccess;
-  if (M == 128 && a.n_pos <= kClusterMax) return launch_cluster(mode, a, st);
+  if (M == 128 && cluster_faster(mode, a, beside)) return launch_cluster(mode, a, st);
   return M == 128 ? launch_m<128>(mode, a, st) : launch_m<64>(mode, a, st);
 }
 

@@ -102,7 +102,8 @@ int chain_threads(int M);
 int chain_blocks_per_sm(int M);  // resident gradient-mode blocks per SM (0 if unknown)
 size_t chain_smem_bytes(int M);
 cudaError_t chain_prepare(int M);  // raise the dynamic shared-memory limit
-cudaError_t launch_chain(int M, ChainMode mode, const ChainArgs& a, cudaStream_t st);
+// beside: waves of positions whose object gradient is accumulated at the same time
+cudaError_t launch_chain(int M, ChainMode mode, const ChainArgs& a, cudaStream_t st, int beside = 0);
 
 // chain_tc.cu (BF16 or F16 hi/lo split DFT products on tcgen05, M = 128)
 size_t chain_tc_smem_bytes();

@@ -510,7 +510,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
     r.loss_part = pl->loss_part + (size_t)off * pl->loss_parts;
     return r;
   };
-  auto launch_chain_for = [&](const ChainArgs& ca) -> int {
+  auto launch_chain_for = [&](const ChainArgs& ca, int beside = 0) -> int {
     int gm_launches = 0;
     if (pl->wv) {
       TIMED(K_CHAIN, 0, launch_chain_gm(mode, ca, pl->wv, p.M, &gm_launches, st));
@@ -519,7 +519,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
     } else if (p.precision != PTYCHO_FP32) {
       TIMED(K_CHAIN, 1, launch_chain_tc(mode, ca, pl->d_cplanes, p.precision == PTYCHO_FP16X3, st));
     } else {
-      TIMED(K_CHAIN, 1, launch_chain(p.M, mode, ca, st));
+      TIMED(K_CHAIN, 1, launch_chain(p.M, mode, ca, st, beside));
     }
     pl->tm.chain_positions += ca.n_pos;
     return PTYCHO_OK;
@@ -606,7 +606,7 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
       }
     } else if (tail) {
       CUDA_TRY(cudaEventRecord(pl->ev_fork, st));
-      if ((rc = launch_chain_for(sub(a, n1, tail))) != PTYCHO_OK) return rc;
+      if ((rc = launch_chain_for(sub(a, n1, tail), n1 / pl->wave)) != PTYCHO_OK) return rc;
       CUDA_TRY(cudaStreamWaitEvent(pl->side, pl->ev_fork, 0));
       if ((rc = accum_for(c0, 0, n1, ci > 0, pl->side)) != PTYCHO_OK) return rc;
       CUDA_TRY(cudaEventRecord(pl->ev_join, pl->side));
