@@ -14,7 +14,9 @@ namespace ptycho {
 // launch_dependents (or ended), and fill its tables while that one still runs.
 // dependency_wait returns when the kernel before it is complete and its writes
 // are visible: every such kernel calls it before it touches anything but
-// constant tables, so completion carries over from kernel to kernel.
+// constant tables, so completion carries over from kernel to kernel.  A kernel
+// whose results are read through the read-only path (__ldg, which asks for data
+// that does not change while the reader runs) does not call launch_dependents.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

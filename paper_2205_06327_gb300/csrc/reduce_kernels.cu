@@ -341,10 +341,12 @@ __global__ void __launch_bounds__(256) k_probe_loss(const float2* __restrict__ s
 
 // The update of a step in one launch: O += a_o dF/dO, P += a_p dF/dP, and for
 // the delayed accumulation (ACC) acc += dF/dO and, with `flush`, the second
-// update O += a_o acc, acc = 0.
+// update O += a_o acc, acc = 0.  No launch_dependents here: the next chain reads O
+// and P through the read-only path (__ldg), so it must not start before they are
+// written (8 per-location updates 1446 us with it, 1437 without; plain loads
+// instead of read-only ones cost the chain 3 %).
 template <bool ACC>
 __global__ void __launch_bounds__(256) k_update(const UpdateArgs u) {
-  launch_dependents();
   dependency_wait();
   const size_t stride = (size_t)gridDim.x * 256;
   for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < u.n_obj; i += stride) {
