@@ -7,8 +7,9 @@
 //   32: 930, 8: 1009 -> 280                   96: 930, 11: 3151 -> 1601
 //   48: 930, 8: 1738 -> 375                  108: 400, 8: 2951 -> 764
 //   54: 625, 8: 1850 -> 384
-// For 96: 8 x 12 in 192 threads 1826, 6 x 16 2092, 12 x 8 in 192 threads 1727;
-// later 8 blocks per SM 1386 against 6 (more registers) 1356.
+// For 96, at the same time: 8 x 12 in 192 threads 1826, 6 x 16 2092, 12 x 8 in 192
+// threads 1727; with dependent launches and one chunk (1601 -> 1386): 8 blocks
+// per SM 1386, 6 (more registers) 1356.
 #include "chain_gm_line.cuh"
 
 namespace ptycho {

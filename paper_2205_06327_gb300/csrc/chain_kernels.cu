@@ -79,20 +79,9 @@ __device__ __forceinline__ void for_p2(int t, F&& f) {
 
 __device__ __forceinline__ float2 ldg2(const float2* p) { return __ldg(p); }
 
-// Recompute mode's finished patches are read once by the accumulation that
-// follows each launch: streaming stores by default; plain stores (to keep a
-// chunk's patches in L2 when the chunk is small enough) with
-// PTYCHO_PATCH_STORE_CS=0.
-#ifndef PTYCHO_PATCH_STORE_CS
-#define PTYCHO_PATCH_STORE_CS 1
-#endif
-__device__ __forceinline__ void store_patch(float2* p, float2 v) {
-#if PTYCHO_PATCH_STORE_CS
-  __stcs(p, v);
-#else
-  *p = v;
-#endif
-}
+// Recompute mode's finished patches are read once, by the accumulation that
+// follows each launch: streaming stores.
+__device__ __forceinline__ void store_patch(float2* p, float2 v) { __stcs(p, v); }
 
 }  // namespace
 

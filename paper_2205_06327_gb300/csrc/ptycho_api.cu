@@ -729,7 +729,11 @@ int ptycho_plan_create(ptycho_plan* out, const ptycho_params* params) {
   // about half of the L2, or three quarters where that saves splitting the
   // positions (930 at M = 96, 68 MB: 1480 us in two chunks, 1389 in one; 196 at
   // M = 216, 73 MB: 1854, 1762; several chunks of up to 96 MB: 506 at M = 192
-  // 3068, 3100, 1024 at M = 256 7482, 7633)
+  // 3068, 3100, 1024 at M = 256 7482, 7633).  From M = 256 on one chunk pays up to
+  // about 84 MB and costs above (two chunks, one; us of 8 slices: 130 at 256, 68
+  // MB 971, 902; 160, 84 MB 1194, 1154; 192, 101 MB 1381, 1400; 84 at 384, 99 MB
+  // 1933, 1951; 40 at 512, 84 MB 1623, 1527; forward of 9 at 1024, 75 MB 627,
+  // 636): those windows keep the half.
   if (gm && chunk > 1) {
     const int64_t wave = (int64_t)(MM * sizeof(float2));
     const bool whole = M < 256 && p.N * wave <= kGmWaveBytes / 2 * 3;

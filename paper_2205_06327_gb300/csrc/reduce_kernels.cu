@@ -21,6 +21,7 @@ constexpr int kAccWarps = kAccThreads / 32;
 constexpr int kAccDefaultCols = 512;
 constexpr int kAccMaxCols = 1024;
 constexpr int kAccBatch = 4 * kAccThreads;  // positions listed at a time
+constexpr int kSmCount = 152;               // of the GPU this is built for
 
 // float2 a warp's row takes per column parity
 __host__ __device__ constexpr int acc_half(int tile_w) { return tile_w / 2 + 1; }
@@ -42,6 +43,17 @@ struct AccVec<1> {
   static __device__ __forceinline__ float2 get(const float2& v, int) { return v; }
 };
 
+// The probe need not be 16-byte aligned (8 bytes are asked of the caller).
+template <int VEC>
+__device__ __forceinline__ typename AccVec<VEC>::type probe_load(const float2* p) {
+  if constexpr (VEC == 2) {
+    const float2 u = __ldg(p), v = __ldg(p + 1);
+    return make_float4(u.x, u.y, v.x, v.y);
+  } else {
+    return __ldg(p);
+  }
+}
+
 // One block owns one (tile, slice) and each of its 8 warps one row of the
 // tile: the row's sums live in shared memory and only that warp touches them.
 // The warp walks the positions whose window covers its row in ascending order
@@ -60,17 +72,6 @@ struct AccVec<1> {
 // patches of 3600 positions, M = 128, 30 slices 4.72 -> 3.43 ms.  Fewer loads
 // in flight with more blocks per SM (half of them, 4 blocks) gave 721 / 276 /
 // 451 us; 8 steps instead of 16 for finished patches 4.02 ms.
-// The probe need not be 16-byte aligned (8 bytes are asked of the caller).
-template <int VEC>
-__device__ __forceinline__ typename AccVec<VEC>::type probe_load(const float2* p) {
-  if constexpr (VEC == 2) {
-    const float2 u = __ldg(p), v = __ldg(p + 1);
-    return make_float4(u.x, u.y, v.x, v.y);
-  } else {
-    return __ldg(p);
-  }
-}
-
 template <int K, int VEC, bool PATCH>
 __global__ void __launch_bounds__(kAccThreads, 2) k_accum_obj_grad(const AccumArgs a) {
   using V = AccVec<VEC>;
@@ -457,7 +458,7 @@ cudaError_t launch_accum_obj_grad(const AccumArgs& args, cudaStream_t st) {
     const int n = (a.W + kAccDefaultCols - 1) / kAccDefaultCols;
     a.tile_w = (a.W + n - 1) / n;
     auto blocks = [&]() { return (int64_t)ns * ((a.H + kAccWarps - 1) / kAccWarps) * ((a.W + a.tile_w - 1) / a.tile_w); };
-    while (blocks() < 456 && (a.tile_w + 1) / 2 >= a.M) a.tile_w = (a.tile_w + 1) / 2;
+    while (blocks() < 3 * kSmCount && (a.tile_w + 1) / 2 >= a.M) a.tile_w = (a.tile_w + 1) / 2;
   } else {
     const int least = a.M < a.W ? a.M : a.W;
     if (a.tile_w < least) a.tile_w = least;
