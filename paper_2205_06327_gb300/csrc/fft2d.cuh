@@ -187,7 +187,7 @@ struct Factors {
   uint32_t tmem;
   const float2* tw1;
   // cluster only: the mbarriers of the two row buffers, the parity of their
-  // next completion, the device error word, and whether this warp still takes
+  // next completion, the device error word, and whether this thread still takes
   // part in the exchanges
   uint64_t* mbar = nullptr;
   uint32_t phase = 0;
@@ -288,26 +288,27 @@ struct ClusterCfg128 : Cfg<128> {
                  "f"(v.x), "f"(v.y), "r"(mbar)
                  : "memory");
   }
-  // Buffer `which`'s exchange number `phase` has arrived.  A warp whose wait
+  // Buffer `which`'s exchange number `phase` has arrived.  A thread whose wait
   // expires reports it and gives up: it neither waits nor arms an mbarrier nor
   // stores into another block from then on (what it computes is meaningless), so
   // the other blocks' next wait expires too and the kernel ends within two
   // limits.  An mbarrier is only armed again by a thread that saw its last phase
   // complete.
   __device__ static __forceinline__ void arrived(Factors& f, int which) {
-    if (f.state & kGaveUp) return;
-    uint64_t* mbar = f.mbar + which;
-    if (threadIdx.x == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(mbar)), "r"(kBytes)
-                   : "memory");
-    const long long limit = f.state & kMuted ? kShortWaitCycles : kWaitCycles;
-    const bool done = tc::mbar_wait_bounded(mbar, f.phase >> which & 1u, limit);
-    if (!__all_sync(0xffffffffu, done)) {
-      *f.status = kWaitExpired;
-      f.state |= kGaveUp;
-      return;
+    if (!(f.state & kGaveUp)) {
+      uint64_t* mbar = f.mbar + which;
+      if (threadIdx.x == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(mbar)), "r"(kBytes)
+                     : "memory");
+      const long long limit = f.state & kMuted ? kShortWaitCycles : kWaitCycles;
+      if (tc::mbar_wait_bounded(mbar, f.phase >> which & 1u, limit)) {
+        f.phase ^= 1u << which;
+      } else {
+        *f.status = kWaitExpired;
+        f.state |= kGaveUp;
+      }
     }
-    f.phase ^= 1u << which;
+    __syncwarp();  // tensor memory is read by whole warps
   }
   // Before a block gives its memory back: no block leaves while another may
   // still store into it.  A block whose exchanges all arrived has nothing in
