@@ -70,9 +70,10 @@ extern "C" {
                                      blocks that share a position (PTYCHO_FP32,
                                      M = 128, few positions), or for the tensor
                                      cores (split precisions).  The call's results
-                                     are meaningless.  Returned by the calls that
-                                     read a scalar on the host (a host loss_out,
-                                     the line search, ptycho_loss_grad_host,
+                                     are meaningless.  Returned (and cleared) by
+                                     the calls that read a scalar on the host (a
+                                     host loss_out, the line search,
+                                     ptycho_loss_grad_host,
                                      ptycho_loss_grad_noalloc), else reported by
                                      ptycho_plan_status after the stream syncs */
 #define PTYCHO_ERR_UNSUPPORTED -6 /* probe window size not supported */

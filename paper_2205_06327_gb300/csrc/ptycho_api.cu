@@ -621,15 +621,18 @@ int run_loss_grad(ptycho_plan pl, const int32_t* pos, const ptycho_c64* probe, c
 }
 
 // The scalars in h_scal, once st is done.  A wait that gave up leaves every
-// number of the call meaningless: a call that reads scalars reports it (the
-// other device errors concern single positions or values and wait for
-// ptycho_plan_status, which reports this one as well).
-int read_scalars(ptycho_plan pl, cudaStream_t st) {
+// number of the call meaningless: a call that reads scalars reports it, and
+// clears the word as ptycho_plan_status does.  The other device errors concern
+// single positions or values; they wait for ptycho_plan_status unless `all`.
+int read_scalars(ptycho_plan pl, cudaStream_t st, bool all = false) {
   CUDA_TRY(cudaMemcpyAsync(pl->h_scal, pl->d_scal, (kStatusSlot + 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   int h;
   std::memcpy(&h, pl->h_scal + kStatusSlot, sizeof h);
-  return h == PTYCHO_ERR_TIMEOUT ? status_fail(h) : PTYCHO_OK;
+  if (!h || (h != PTYCHO_ERR_TIMEOUT && !all)) return PTYCHO_OK;
+  CUDA_TRY(cudaMemsetAsync(pl->d_status, 0, sizeof(int), st));
+  CUDA_TRY(cudaStreamSynchronize(st));
+  return status_fail(h);
 }
 
 int deliver_loss(ptycho_plan pl, int slot, double* loss_out, cudaStream_t st) {
@@ -1224,18 +1227,10 @@ int loss_grad_host_impl(ptycho_plan plan, const int32_t* pos_yx, const ptycho_c6
   }
   if (grad_obj) CUDA_TRY(cudaMemcpyAsync(grad_obj, pl->x_gO, sizeof(float2) * nO, cudaMemcpyDeviceToHost, st));
   if (grad_probe) CUDA_TRY(cudaMemcpyAsync(grad_probe, pl->x_gP, sizeof(float2) * MM, cudaMemcpyDeviceToHost, st));
-  // The call is synchronous, so it reports the device error word itself (and clears it).
-  rc = read_scalars(pl, st);
-  if (rc && rc != PTYCHO_ERR_TIMEOUT) return rc;
-  *loss_out = pl->h_scal[0];
-  int h;
-  std::memcpy(&h, pl->h_scal + kStatusSlot, sizeof h);
-  if (h) {
-    CUDA_TRY(cudaMemsetAsync(pl->d_status, 0, sizeof(int), st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    return status_fail(h);
-  }
-  return PTYCHO_OK;
+  // The call is synchronous, so it reports the device error word itself.
+  rc = read_scalars(pl, st, true);
+  if (rc != PTYCHO_ERR_CUDA) *loss_out = pl->h_scal[0];
+  return rc;
 }
 
 }  // namespace
